@@ -40,6 +40,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "chem_internal.h"
 
 namespace chem {
@@ -52,7 +54,16 @@ enum SlotState : int {
     kNewtonT = 2,     // needs the temperature of the current Newton iterate
     kNewtonReady = 3, // runs a Newton iteration this trip
     kCheckT = 4,      // needs the temperature of a converged iterate
-    kDead = 5         // no more cells
+    kRejected = 5,    // its substep attempt failed
+    kDead = 6         // no more cells
+};
+// What a slot's settled state asks for, done in one place per pass (each
+// copy of that code would take its share of the instruction caches).
+enum SlotAction : int {
+    kNoAction = 0,
+    kStartSubstep = 1,
+    kFailSubstep = 2,
+    kEmitCell = 3
 };
 
 template <int G>
@@ -472,6 +483,180 @@ __device__ __forceinline__ void lu_update_colmajor(float *A, int ld, int n, int 
     }
 }
 
+// FP32 elimination of [A | rhs] and back substitution with the matrix in
+// registers (one cell per warp, kLuRegMinN <= N <= kLuRegN unknowns).  Lane l
+// holds row l, one column per register; the rows past 32 (at most four) are
+// spread over eight lanes each.  Rows never move: id0 (and id1 of the lane's
+// row past 32) carries the index the row would have after the swaps, and is
+// negative once the row has been a pivot.  Step j: two redux find the pivot
+// (largest |a_ij|, then the lowest index), its owner writes the row's columns
+// j .. N to shared memory (row j of U, from A's start on), and every lane
+// reads them back and updates its rows with fma(-a_ij, a_jk / a_jj, a_ik): the
+// pivots and roundings of lu_update_colmajor.  The results move one register
+// down, so that column j is always in register 0 and the loop body is one
+// copy of the code.  The solution goes to A[N ld ...].
+//   Bound by latency.  A branch costs a warp some thirty cycles here, so the
+// body is straight-line: registers past the live columns are carried along
+// (what they hold is never used), rows of U may run past their end into the
+// next row's place, and only whole groups of eight columns are skipped.
+constexpr int kLuRegMinN = 24, kLuRegN = 36;
+// floats of U's rows of length 1 .. L (columns j .. N, rounded up to 4)
+__device__ __forceinline__ int lu_u_size(int L) {
+    const int q = L >> 2, r = L & 3;
+    return (8 * q + 4 * r) * (q + 1);
+}
+__device__ __forceinline__ bool lu_registers(float *A, int ld, int N, int lane) {
+    constexpr int NC = 40, NE = 5;
+    float a[NC], x[NE];
+    const int xr = 32 + (lane >> 3), xc = lane & 7;   // the lane's row past 32, its columns 8 q + xc
+    const bool extra = N > 32;
+    const int li = min(lane, N - 1);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) a[k] = A[min(k, N) * ld + li];
+    int id0 = lane < N ? lane << 8 | lane : -1, id1 = xr < N ? xr << 8 | xr : -1;
+#pragma unroll
+    for (int q = 0; q < NE; ++q) x[q] = A[min(8 * q + xc, N) * ld + min(xr, N - 1)];
+    __syncwarp();   // every entry is in a register before U's rows are stored
+    unsigned worst = 0x7f7fffffu, most = 0u;   // smallest and largest pivot key
+    float *u = A;   // row j of U: columns j .. N
+#pragma unroll 1
+    for (int j = 0; j < N; ++j) {
+        const int cols = N + 1 - j, xo = xc - (j & 7);   // xo: offset in u of the lane's slot 0
+        const float m0 = a[0], m1 = __shfl_sync(kFull, x[0], (lane & ~7) | (j & 7));
+        const unsigned k0 = abs_key(m0), k1 = abs_key(m1);
+        const unsigned best = __reduce_max_sync(kFull, max(id0 >= 0 ? k0 : 0u, id1 >= 0 ? k1 : 0u));
+        // (the index of a row that is done is above any as an unsigned number)
+        const unsigned cand = __reduce_min_sync(kFull, min(k0 == best ? (unsigned)id0 : 0xffffffffu,
+                                                           k1 == best ? (unsigned)id1 : 0xffffffffu));
+        worst = min(worst, best);
+        most = max(most, best);
+        const bool p0 = id0 == (int)cand, p1 = id1 == (int)cand;
+        if (p0) {
+#pragma unroll
+            for (int c = 0; c < NC; c += 8) {
+                if (c >= cols) break;
+                *reinterpret_cast<float4 *>(u + c) = make_float4(a[c], a[c + 1], a[c + 2], a[c + 3]);
+                *reinterpret_cast<float4 *>(u + c + 4) = make_float4(a[c + 4], a[c + 5], a[c + 6], a[c + 7]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NE; ++q)
+            if (p1 && 8 * q + xo >= 0) u[8 * q + xo] = x[q];
+        // the row at index j takes the pivot's index
+        const int cp = (int)(cand & 0xffffff00u);
+        id0 = p0 ? -1 : id0 >> 8 == j ? cp | (id0 & 0xff) : id0;
+        id1 = p1 ? -1 : id1 >> 8 == j ? cp | (id1 & 0xff) : id1;
+        __syncwarp();
+        const float inv = frcp(u[0]);
+        if (extra) {
+#pragma unroll
+            for (int q = 0; q < NE; ++q) x[q] = fmaf(-m1, u[max(8 * q + xo, 0)] * inv, x[q]);
+            if ((j & 7) == 7) {
+#pragma unroll
+                for (int q = 0; q + 1 < NE; ++q) x[q] = x[q + 1];
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NC; c += 8) {
+            if (c >= cols) break;
+            const float4 v = *reinterpret_cast<const float4 *>(u + c), w = *reinterpret_cast<const float4 *>(u + c + 4);
+            if (c > 0) a[c - 1] = fmaf(-m0, v.x * inv, a[c]);
+            a[c] = fmaf(-m0, v.y * inv, a[c + 1]);
+            a[c + 1] = fmaf(-m0, v.z * inv, a[c + 2]);
+            a[c + 2] = fmaf(-m0, v.w * inv, a[c + 3]);
+            a[c + 3] = fmaf(-m0, w.x * inv, a[c + 4]);
+            a[c + 4] = fmaf(-m0, w.y * inv, a[c + 5]);
+            a[c + 5] = fmaf(-m0, w.z * inv, a[c + 6]);
+            a[c + 6] = fmaf(-m0, w.w * inv, a[c + 7]);
+        }
+        u += (cols + 3) & ~3;
+    }
+    // back substitution: lane l solves rows l and l + 32; each solved entry
+    // reaches the lanes by a shuffle
+    const int n1 = lu_u_size(N + 1), l1 = min(lane + 32, N - 1);
+    const float *u0 = A + (n1 - lu_u_size(N + 1 - li) - li), *u1 = A + (n1 - lu_u_size(N + 1 - l1) - l1);
+    float y0 = u0[N], y1 = u1[N];
+    const float d0 = frcp(u0[li]), d1 = frcp(u1[l1]);
+#pragma unroll 1
+    for (int j = N - 1; j >= 32; --j) {
+        const float v0 = u0[j], v1 = u1[j];
+        const float dj = __shfl_sync(kFull, y1 * d1, j & 31);
+        y0 = fmaf(-v0, dj, y0);
+        y1 = lane + 32 < j ? fmaf(-v1, dj, y1) : lane + 32 == j ? dj : y1;
+    }
+#pragma unroll 2
+    for (int j = min(N, 32) - 1; j >= 0; --j) {
+        const float v0 = u0[j];
+        const float dj = __shfl_sync(kFull, y0 * d0, j);
+        y0 = lane < j ? fmaf(-v0, dj, y0) : lane == j ? dj : y0;
+    }
+    __syncwarp();
+    if (lane < N) A[N * ld + lane] = y0;
+    if (lane + 32 < N) A[N * ld + lane + 32] = y1;
+    __syncwarp();
+    return worst == 0u || key_is_inf(most);
+}
+
+// The elimination by columns and the back substitution of one cell per warp
+// for the sizes lu_registers does not take.  Out of line, so that it takes no
+// place in the instruction caches beside the code that runs.
+static __device__ __noinline__ bool lu_columns(unsigned A_shared, int ld, int N) {
+    float *A = static_cast<float *>(__cvta_shared_to_generic(A_shared));
+    const int lane = threadIdx.x & 31;
+    bool sing = false;
+#pragma unroll 1
+    for (int j = 0; j < N; ++j) {
+        unsigned best = 0;
+        int bi = N;
+#pragma unroll 1
+        for (int i = j + lane; i < N; i += 32) {
+            const unsigned kk = abs_key(A[j * ld + i]);
+            if (bi == N || kk > best) {
+                best = kk;
+                bi = i;
+            }
+        }
+        warp_argmax(best, bi);
+        if (best == 0 || key_is_inf(best)) sing = true;
+        if (bi != j && bi < N) {
+#pragma unroll 1
+            for (int k = j + lane; k <= N; k += 32) {
+                const float t = A[k * ld + j];
+                A[k * ld + j] = A[k * ld + bi];
+                A[k * ld + bi] = t;
+            }
+        }
+        __syncwarp();
+        const float inv = frcp(A[j * ld + j]);
+        lu_update_colmajor<32>(A, ld, N, j, lane, inv);
+        __syncwarp();
+        // the reciprocal replaces the pivot once every lane has read it
+        if (lane == 0) A[j * ld + j] = inv;
+    }
+    __syncwarp();
+    // lane l keeps rows l and l + 32 of the right-hand side in registers, and
+    // each solved entry reaches the lanes by a shuffle
+    float y0 = lane < N ? A[N * ld + lane] : 0.f, y1 = lane + 32 < N ? A[N * ld + lane + 32] : 0.f;
+#pragma unroll 1
+    for (int j = N - 1; j >= 0; --j) {
+        const float yj = __shfl_sync(kFull, j < 32 ? y0 : y1, j & 31);
+        const float dj = yj * A[j * ld + j];
+        if (lane == (j & 31)) {
+            if (j < 32)
+                y0 = dj;
+            else
+                y1 = dj;
+        }
+        if (lane < j) y0 = fmaf(-A[j * ld + lane], dj, y0);
+        if (lane + 32 < j) y1 = fmaf(-A[j * ld + lane + 32], dj, y1);
+    }
+    __syncwarp();
+    if (lane < N) A[N * ld + lane] = y0;
+    if (lane + 32 < N) A[N * ld + lane + 32] = y1;
+    __syncwarp();
+    return sing;
+}
+
 template <typename JT>
 struct SlotMem {
     double *x, *x0, *c, *hRT, *es, *em, *emi, *Q, *part;
@@ -727,23 +912,56 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     //    (an item's partial sums: sum nu Q in FP64, then sum nu dQ/dT and
     //    sum nu q_tb in the Jacobian type, packed into the next 16 bytes)
     const GatherLayout &gl = m.gl[layout_index(G)];
+    //   The table's words come from L2 as often as from L1, so an item's
+    //   eight words are loaded together, the next item's descriptor with
+    //   them, and the operands of four terms at a time; the sums keep the
+    //   order of the list.
+    auto item_at = [&](int it) -> int2 { return it < m.n_items ? __ldg(gl.it_meta + it) : make_int2(0, 0); };
+    auto item_words = [&](int e, int rem) -> uint4 {
+        const unsigned *wp = gl.sp_w + e;
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (rem > 0) w.x = __ldg(wp);
+        if (rem > 1) w.y = __ldg(wp + G);
+        if (rem > 2) w.z = __ldg(wp + 2 * G);
+        if (rem > 3) w.w = __ldg(wp + 3 * G);
+        return w;
+    };
+    static_assert(kChunk == 8, "an item is two groups of four terms");
+    int2 im = item_at(sl);
+    uint4 iwords = item_words(im.x, im.y);
 #pragma unroll 1
     for (int it = sl; it < m.n_items; it += G) {
-        const int2 im = __ldg(gl.it_meta + it);
+        const int e1 = im.x + 4 * G;
+        int rem = im.y;
+        im = item_at(it + G);
         double sq = 0.0;
         JT sdq = 0, squ = 0;
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            const uint4 wc = iwords;
+            iwords = half == 0 ? item_words(e1, rem - 4) : item_words(im.x, im.y);
+            const unsigned wv[4] = {wc.x, wc.y, wc.z, wc.w};
+            double Qv[4];
+            JT dq[4], qt[4];
 #pragma unroll
-        for (int q = 0; q < kChunk; ++q) {
-            if (q < im.y) {
-                const int e = im.x + q * G;
-                const unsigned wv = __ldg(gl.sp_w + e);
-                const int r = (int)(wv & 0xfffffu);
-                const double nu = word_nu_double(wv);   // nu_rs != 0 in a list
-                const JT nuj = f32 ? (JT)word_nu_float(wv) : (JT)nu;
-                sq = fma(nu, sm.Q[r], sq);
-                sdq += nuj * sm.dQdT[r];
-                if (r < m.ntb) squ += nuj * sm.qtb[r];
+            for (int q = 0; q < 4; ++q) {
+                // (a missing term's word is 0: reaction 0 is read and not used)
+                const int r = (int)(wv[q] & 0xfffffu);
+                Qv[q] = sm.Q[r];
+                dq[q] = sm.dQdT[r];
+                qt[q] = r < m.ntb ? sm.qtb[r] : (JT)0;
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (q < rem) {
+                    const double nu = word_nu_double(wv[q]);   // nu_rs != 0 in a list
+                    const JT nuj = f32 ? (JT)word_nu_float(wv[q]) : (JT)nu;
+                    sq = fma(nu, Qv[q], sq);
+                    sdq += nuj * dq[q];
+                    if ((int)(wv[q] & 0xfffffu) < m.ntb) squ += nuj * qt[q];
+                }
+            }
+            rem -= 4;
         }
         constexpr int iw = (int)(item_bytes((int)sizeof(JT)) / 8);   // doubles per item
         sm.part[iw * it] = sq;
@@ -896,57 +1114,117 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         //     added as -h (M_s / M_k) sum_r nu_rs D_rk
         //     (the word's top nine bits are those of the float coefficient)
         auto coef = [](unsigned wv) -> float { return __int_as_float((int)(wv & 0xff800000u)); };
+        //     Most lists have fewer than four terms, and the table's words
+        //     often come from L2: a list's metadata is loaded two entries
+        //     ahead, its first four words one entry ahead, later words one
+        //     chunk ahead, and a chunk's terms are read together.  Terms in
+        //     a whole chunk alternate between two accumulators, those of a
+        //     partial one follow the first.
+        const int nnz = m.nJ_nz;
+        auto meta_at = [&](int p) -> int4 { return p < nnz ? __ldg(gl.j_meta32 + p) : make_int4(0, 0, 0, 0); };
+        auto words_at = [&](int e, int rem) -> uint4 {
+            const unsigned *wp = gl.j_w + e;
+            uint4 w = make_uint4(0u, 0u, 0u, 0u);
+            if (rem > 0) w.x = __ldg(wp);
+            if (rem > 1) w.y = __ldg(wp + G);
+            if (rem > 2) w.z = __ldg(wp + 2 * G);
+            if (rem > 3) w.w = __ldg(wp + 3 * G);
+            return w;
+        };
+        int4 me = meta_at(sl), mn = meta_at(sl + G);
+        uint4 wn = words_at(me.x, me.y);
 #pragma unroll 1
-        for (int p = sl; p < m.nJ_nz; p += G) {
-            const int4 meta = __ldg(gl.j_meta32 + p);
-            const int len = meta.y;
+        for (int p = sl; p < nnz; p += G) {
+            float *ap = reinterpret_cast<float *>(sm.A) + me.z;
+            const float av = *ap, fac = mh * __int_as_float(me.w);
+            int e = me.x, rem = me.y;
+            uint4 w = wn;
+            me = mn;
+            mn = meta_at(p + 2 * G);
+            wn = words_at(me.x, me.y);
             float a0 = 0.f, a1 = 0.f;
-            int e = meta.x, q = 0;
 #pragma unroll 1
-            for (; q + 4 <= len; q += 4, e += 4 * G) {
-                const unsigned w0 = __ldg(gl.j_w + e), w1 = __ldg(gl.j_w + e + G), w2 = __ldg(gl.j_w + e + 2 * G),
-                               w3 = __ldg(gl.j_w + e + 3 * G);
-                const float v0 = Dv[w0 & 0x7fffffu], v1 = Dv[w1 & 0x7fffffu], v2 = Dv[w2 & 0x7fffffu],
-                            v3 = Dv[w3 & 0x7fffffu];
-                a0 = fmaf(coef(w0), v0, a0);
-                a1 = fmaf(coef(w1), v1, a1);
-                a0 = fmaf(coef(w2), v2, a0);
-                a1 = fmaf(coef(w3), v3, a1);
+            for (;;) {
+                // (a missing term's word is 0: D entry 0 is read and not used)
+                const float v0 = Dv[w.x & 0x7fffffu], v1 = Dv[w.y & 0x7fffffu], v2 = Dv[w.z & 0x7fffffu],
+                            v3 = Dv[w.w & 0x7fffffu];
+                const uint4 wc = w;
+                const int rc = rem;
+                rem -= 4;
+                e += 4 * G;
+                w = words_at(e, rem);
+                if (rc >= 4) {
+                    a0 = fmaf(coef(wc.x), v0, a0);
+                    a1 = fmaf(coef(wc.y), v1, a1);
+                    a0 = fmaf(coef(wc.z), v2, a0);
+                    a1 = fmaf(coef(wc.w), v3, a1);
+                } else {
+                    a0 = fmaf(coef(wc.x), v0, a0);
+                    if (rc > 1) a0 = fmaf(coef(wc.y), v1, a0);
+                    if (rc > 2) a0 = fmaf(coef(wc.z), v2, a0);
+                }
+                if (rem <= 0) break;
             }
-#pragma unroll 1
-            for (; q < len; ++q, e += G) {
-                const unsigned wv = __ldg(gl.j_w + e);
-                a0 = fmaf(coef(wv), Dv[wv & 0x7fffffu], a0);
-            }
-            float *ap = reinterpret_cast<float *>(sm.A) + meta.z;
-            *ap = fmaf(mh * __int_as_float(meta.w), a0 + a1, *ap);
+            *ap = fmaf(fac, a0 + a1, av);
         }
         __syncwarp();
     } else {
+        // (loads ahead as in the FP32 pass; an addition whose operand is an
+        // exact zero costs an FP64-pipe slot like any other and is skipped)
+        struct Terms {
+            int d[4];
+            double c[4];
+        };
+        auto terms_at = [&](int e, int rem) -> Terms {
+            Terms t;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                t.d[i] = rem > i ? __ldg(gl.j_d + e + i * G) : 0;
+                t.c[i] = rem > i ? __ldg(gl.j_c + e + i * G) : 0.0;
+            }
+            return t;
+        };
+        auto meta_at = [&](int p) -> int2 { return p < m.nJ ? __ldg(gl.j_meta + p) : make_int2(0, 0); };
+        int2 me = meta_at(sl), mn = meta_at(sl + G);
+        Terms tn = terms_at(me.x, me.y >> 16);
 #pragma unroll 1
         for (int p = sl; p < m.nJ; p += G) {
-            const int2 meta = __ldg(gl.j_meta + p);
-            const int len = meta.y >> 16;
-            const int s = (meta.y >> 8) & 0xff, k = meta.y & 0xff;
+            const int len = me.y >> 16, s = (me.y >> 8) & 0xff, k = me.y & 0xff;
+            int e = me.x, rem = len;
+            Terms t = tn;
+            me = mn;
+            mn = meta_at(p + 2 * G);
+            tn = terms_at(me.x, me.y >> 16);
             const JT invMk = (JT)__ldg(m.sp + k * kSpStride + 1);
-            JT J = sm.w[s] * sm.dTdr[k];
-            JT a0 = 0, a1 = 0;
-            int e = meta.x, q = 0;
+            const JT J = sm.w[s] * sm.dTdr[k];
+            JT ua = sm.u[s];
+            if (len > 0) {
+                JT a0 = 0, a1 = 0;
 #pragma unroll 1
-            for (; q + 4 <= len; q += 4, e += 4 * G) {
-                const int d0 = __ldg(gl.j_d + e), d1 = __ldg(gl.j_d + e + G), d2 = __ldg(gl.j_d + e + 2 * G),
-                          d3 = __ldg(gl.j_d + e + 3 * G);
-                const JT v0 = Dv[d0], v1 = Dv[d1], v2 = Dv[d2], v3 = Dv[d3];
-                a0 = fma((JT)__ldg(gl.j_c + e), v0, a0);
-                a1 = fma((JT)__ldg(gl.j_c + e + G), v1, a1);
-                a0 = fma((JT)__ldg(gl.j_c + e + 2 * G), v2, a0);
-                a1 = fma((JT)__ldg(gl.j_c + e + 3 * G), v3, a1);
+                for (;;) {
+                    const JT v0 = Dv[t.d[0]], v1 = Dv[t.d[1]], v2 = Dv[t.d[2]], v3 = Dv[t.d[3]];
+                    const Terms tc = t;
+                    const int rc = rem;
+                    rem -= 4;
+                    e += 4 * G;
+                    t = terms_at(e, rem);
+                    if (rc >= 4) {
+                        a0 = fma((JT)tc.c[0], v0, a0);
+                        a1 = fma((JT)tc.c[1], v1, a1);
+                        a0 = fma((JT)tc.c[2], v2, a0);
+                        a1 = fma((JT)tc.c[3], v3, a1);
+                    } else {
+                        a0 = fma((JT)tc.c[0], v0, a0);
+                        if (rc > 1) a0 = fma((JT)tc.c[1], v1, a0);
+                        if (rc > 2) a0 = fma((JT)tc.c[2], v2, a0);
+                    }
+                    if (rem <= 0) break;
+                }
+                if (len >= 4) a0 += a1;
+                ua += a0;
             }
-#pragma unroll 1
-            for (; q < len; ++q, e += G) a0 = fma((JT)__ldg(gl.j_c + e), Dv[__ldg(gl.j_d + e)], a0);
             // (D entries scaled by M_k; the FP64 lists' coefficients are nu_rs M_s)
-            J = fma(invMk, sm.u[s] + (a0 + a1), J);
-            sm.A[ix(s, k)] = mh * J;
+            sm.A[ix(s, k)] = mh * fma(invMk, ua, J);
         }
         __syncwarp();
 #pragma unroll 1
@@ -958,6 +1236,11 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     //    (Sec. 3.2), ties to the lowest row; the pivot's reciprocal replaces
     //    the diagonal
     bool sing = false;
+    if constexpr (f32 && G == 32) {
+        sing = N >= kLuRegMinN && N <= kLuRegN
+                   ? lu_registers(reinterpret_cast<float *>(sm.A), ldc, N, sl)
+                   : lu_columns((unsigned)__cvta_generic_to_shared(sm.A), ldc, N);
+    } else {
 #pragma unroll 1
     for (int j = 0; j < N; ++j) {
         PivotKey<JT> best = 0;
@@ -1028,30 +1311,6 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     }
     __syncwarp();
     // back substitution, U delta = y
-    if constexpr (f32 && G == 32) {
-        // one cell per warp (N <= 64): lane l keeps rows l and l + 32 of the
-        // right-hand side in registers, and each solved entry reaches the
-        // lanes by a shuffle instead of shared memory and two warp barriers
-        // (the FP64 path measured 1 % slower this way)
-        JT y0 = sl < N ? sm.A[ix(sl, N)] : JT(0), y1 = sl + 32 < N ? sm.A[ix(sl + 32, N)] : JT(0);
-#pragma unroll 1
-        for (int j = N - 1; j >= 0; --j) {
-            const JT yj = __shfl_sync(kFull, j < 32 ? y0 : y1, j & 31);
-            const JT dj = yj * sm.A[ix(j, j)];
-            if (sl == (j & 31)) {
-                if (j < 32)
-                    y0 = dj;
-                else
-                    y1 = dj;
-            }
-            if (sl < j) y0 = fma(-sm.A[ix(sl, j)], dj, y0);
-            if (sl + 32 < j) y1 = fma(-sm.A[ix(sl + 32, j)], dj, y1);
-        }
-        __syncwarp();
-        if (sl < N) sm.A[ix(sl, N)] = y0;
-        if (sl + 32 < N) sm.A[ix(sl + 32, N)] = y1;
-        __syncwarp();
-    } else {
 #pragma unroll 1
         for (int j = N - 1; j >= 0; --j) {
             const JT dj = sm.A[ix(j, N)] * sm.A[ix(j, j)];
@@ -1352,34 +1611,6 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
             }
         }
     };
-    auto write_fail = [&](int code) {
-        emit(code, Tin);
-        state = kFree;
-    };
-    auto start_substep = [&]() {
-        if (attempts >= o.max_attempts) {
-            write_fail(kCellTooManySteps);
-            return;
-        }
-        while ((total >> level) > total - t_units) ++level;
-        h = ldexp(sdt, -level);
-        ++attempts;
-#pragma unroll 1
-        for (int i = sl; i < n; i += G) sm.x[i] = sm.x0[i];
-        T = T0;
-        k = 0;
-        norm_prev = CUDART_INF;
-        state = kNewtonReady;
-    };
-    auto substep_fail = [&]() {
-        ++fails;
-        ++level;
-        if (level > o.max_halvings)
-            write_fail(kCellNewtonFailed);
-        else
-            start_substep();
-    };
-
 #pragma unroll 1
     for (;;) {
         // refill free slots and settle every pending temperature recovery
@@ -1436,6 +1667,8 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
                 if (state == kFree && !loading) state = kDead;
                 if (loading) cell = got;
             }
+            int act = state == kRejected ? kFailSubstep : kNoAction, code = kCellOk;
+            bool advanced = false;   // the cell reached dt: its state is written
             int nonfin = 0;
             double rt = 0.0, es = 0.0;
             if (loading) {
@@ -1466,14 +1699,16 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
                 atol_rho = o.atol_rel * rt;
                 atol_e = o.atol_rel * es;
                 T = (!Q && b.T_in) ? b.T_in[cell] : 1500.0;
-                if (nonfin || !(rt > 0.0))
-                    write_fail(kCellBadInput);
-                else
+                if (nonfin || !(rt > 0.0)) {
+                    act = kEmitCell;
+                    code = kCellBadInput;
+                } else {
                     state = kInitT;
+                }
             }
             __syncwarp();
             const bool needT = state == kInitT || state == kNewtonT || state == kCheckT;
-            if (!__any_sync(kFull, needT)) break;
+            if (!__any_sync(kFull, needT || act != kNoAction)) break;
             double Tr = T;
             bool ok = false;
             recover_T<G, sizeof(JT) == 4>(m, sm.x, sl, needT, T, Tr, ok);
@@ -1485,29 +1720,25 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
             __syncwarp();
             if (state == kInitT) {
                 if (!ok) {
-                    write_fail(kCellTFailed);
+                    act = kEmitCell;
+                    code = kCellTFailed;
                 } else {
                     T = T0 = Tin = Tr;
-                    if (sdt == 0.0) {
-                        emit(kCellOk, Tr);
-                        state = kFree;
-                    } else {
-                        t_units = 0;
-                        level = 0;
-                        attempts = 0;
-                        start_substep();
-                    }
+                    t_units = 0;
+                    level = 0;
+                    attempts = 0;
+                    act = sdt == 0.0 ? kEmitCell : kStartSubstep;
                 }
             } else if (state == kNewtonT) {
                 if (!ok) {
-                    substep_fail();
+                    act = kFailSubstep;
                 } else {
                     T = Tr;
                     state = kNewtonReady;
                 }
             } else if (state == kCheckT) {
                 if (!ok || neg) {
-                    substep_fail();
+                    act = kFailSubstep;
                 } else {
                     T = Tr;
                     // accept the substep (and record it: attempt attempts - 1
@@ -1527,33 +1758,60 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
                     t_units += total >> level;
                     ++subs;
                     if (level > 0) --level;
-                    if (t_units == total) {
-                        double *rho_out = b.rho, *e_out = b.e;
-                        long long ld_out = b.ld;
-                        if constexpr (Q) {
-                            const ServeDesc *d = b.queue.mdesc + qe;
-                            rho_out = ld_cg(&d->rho);
-                            e_out = ld_cg(&d->e);
-                            ld_out = ld_cg(&d->ld);
-                        }
+                    advanced = t_units == total;
+                    act = advanced ? kEmitCell : kStartSubstep;
+                }
+            }
+            if (act == kFailSubstep) {
+                ++fails;
+                ++level;
+                act = kStartSubstep;
+                if (level > o.max_halvings) {
+                    act = kEmitCell;
+                    code = kCellNewtonFailed;
+                }
+            }
+            if (act == kStartSubstep) {
+                if (attempts >= o.max_attempts) {
+                    act = kEmitCell;
+                    code = kCellTooManySteps;
+                } else {
+                    while ((total >> level) > total - t_units) ++level;
+                    h = sdt * __hiloint2double((1023 - level) << 20, 0);   // sdt 2^-level, level <= 40
+                    ++attempts;
 #pragma unroll 1
-                        for (int i = sl; i < n; i += G) {
-                            if (i < ns)
-                                rho_out[(size_t)i * ld_out + cell] = sm.x[i];
-                            else
-                                e_out[cell] = sm.x[i];
-                        }
-                        if constexpr (Q) {
-                            // every lane's results before lane 0 counts the cell done
-                            // (the slot's G lanes are converged here)
-                            __syncwarp(G == 32 ? kFull : (((1u << G) - 1u) << (slot * G)));
-                        }
-                        emit(kCellOk, T);
-                        state = kFree;
-                    } else {
-                        start_substep();
+                    for (int i = sl; i < n; i += G) sm.x[i] = sm.x0[i];
+                    T = T0;
+                    k = 0;
+                    norm_prev = CUDART_INF;
+                    state = kNewtonReady;
+                }
+            }
+            if (act == kEmitCell) {
+                if (advanced) {
+                    double *rho_out = b.rho, *e_out = b.e;
+                    long long ld_out = b.ld;
+                    if constexpr (Q) {
+                        const ServeDesc *d = b.queue.mdesc + qe;
+                        rho_out = ld_cg(&d->rho);
+                        e_out = ld_cg(&d->e);
+                        ld_out = ld_cg(&d->ld);
+                    }
+#pragma unroll 1
+                    for (int i = sl; i < n; i += G) {
+                        if (i < ns)
+                            rho_out[(size_t)i * ld_out + cell] = sm.x[i];
+                        else
+                            e_out[cell] = sm.x[i];
+                    }
+                    if constexpr (Q) {
+                        // every lane's results before lane 0 counts the cell done
+                        // (the slot's G lanes are converged here)
+                        __syncwarp(G == 32 ? kFull : (((1u << G) - 1u) << (slot * G)));
                     }
                 }
+                emit(code, code == kCellOk ? T : Tin);
+                state = kFree;
             }
             __syncwarp();
         }
@@ -1585,24 +1843,20 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
             // start the next temperature recovery from the linear prediction
             if (bits_gt(T_pred, kTlo) && bits_lt(T_pred, kThi)) T = T_pred;
             ++iters;
-            if (bad) {
-                substep_fail();
-            } else if (o.point_implicit || !bits_gt(norm, 1.0) ||
-                       (o.conv_kappa > 0.0 && k >= 1 && bits_lt(norm, norm_prev) &&
-                        norm * norm <= o.conv_kappa * (norm_prev - norm))) {
+            if (o.point_implicit || !bits_gt(norm, 1.0) ||
+                (o.conv_kappa > 0.0 && k >= 1 && bits_lt(norm, norm_prev) &&
+                 norm * norm <= o.conv_kappa * (norm_prev - norm))) {
                 // (the contraction-rate stop theta / (1 - theta) norm <= kappa,
                 // theta = norm / norm_prev < 1, multiplied out: no division)
                 state = kCheckT;
             } else if (o.div_check && k >= 2 && !bits_lt(norm, norm_prev)) {
-                substep_fail();
+                state = kRejected;
             } else {
                 norm_prev = norm;
                 ++k;
-                if (k >= o.max_newton)
-                    substep_fail();
-                else
-                    state = kNewtonT;
+                state = k >= o.max_newton ? kRejected : kNewtonT;
             }
+            if (bad) state = kRejected;
         }
         __syncwarp();
     }
