@@ -168,9 +168,9 @@ struct HostTables {
     std::vector<unsigned> div16;
     std::vector<float> tpoly_f;
     std::vector<float> rxn_df, d_cef, spf;
-    std::vector<int2> d_pk;
+    std::vector<int2> d_pk, d_pk64;
     std::vector<unsigned> j_w, sp_w;
-    std::vector<int> rxn_f, eff_ptr, eff_sp, d_i0, d_i1, j_sk, j_ptr, j_d, it_ptr, sp_item_ptr, sp_r;
+    std::vector<int> rxn_f, eff_ptr, eff_sp, d_i0, d_i1, j_sk, j_ptr, j_d, it_ptr, it_id, sp_item_ptr, sp_r;
     std::vector<int2> j_meta;
     std::vector<int> j_nu, sp_nui, j_sk32, j_ptr32, j_d32;
     struct Layout {
@@ -180,7 +180,7 @@ struct HostTables {
         std::vector<int> j_d;
         std::vector<double> j_c;
     } lay[kLayouts];
-    int nD = 0, nD_F = 0, nD_B = 0, nD_FB = 0, nJ = 0, nJ_nz = 0, n_items = 0, ntb = 0;
+    int nD = 0, nD_F1 = 0, nD_B1 = 0, nJ = 0, nJ_nz = 0, n_items = 0, ntb = 0;
 };
 
 // {1/F, ln F} at F = 1 + j/kLogTab, j = 0..kLogTab, rounded from extended
@@ -192,6 +192,19 @@ void fill_log_table(std::vector<double> &tab) {
         tab[2 * j] = (double)(1.0L / F);
         tab[2 * j + 1] = (double)std::log(F);
     }
+}
+
+// 2^(j/kExpTab), rounded from extended precision, and the constants that
+// follow it (chem_internal.h)
+void fill_exp_table(std::vector<double> &tab) {
+    tab.resize(kExpTabSize);
+    for (int j = 0; j < kExpTab; ++j) tab[j] = (double)std::exp2l((long double)j / kExpTab);
+    const double c[kExpTabSize - kExpTab] = {1.0, -0.0,
+                                             369.3299304675746, 6755399441055744.0,
+                                             -0x1.62e42fefa0000p-9, -0x1.cf79abc9e3b3ap-48,
+                                             1.0 / 24.0, 1.0 / 6.0, 0.5, 1.0,
+                                             -1.0 / 6.0, 0.2, -0.25, 1.0 / 3.0, -0.5, 0.6931471805599453};
+    std::copy(c, c + (kExpTabSize - kExpTab), tab.begin() + kExpTab);
 }
 
 static void build_tables(const chem_mech_desc *d, HostTables &t) {
@@ -328,12 +341,24 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
     std::stable_sort(ents.begin(), ents.end(), [](const DEnt &a, const DEnt &b) { return a.grp < b.grp; });
     t.nD = (int)ents.size();
     for (const auto &e : ents) {
-        if (e.grp <= 0) t.nD_F++;
-        if (e.grp <= 1) t.nD_B++;
-        if (e.grp <= 2) t.nD_FB++;
         t.d_i0.push_back(e.r | (e.vf << 16) | (e.vb << 20));
         t.d_cef.push_back((float)e.alpha1);
         t.d_i1.push_back(e.fa | (e.fb << 8) | (e.ba << 16) | (e.bb << 24));
+    }
+    // the FP64 kernel's order: entries that take one multiplication first
+    auto kind64 = [&](const DEnt &e) {
+        const bool one = e.vf + e.vb == 1 && (e.vf ? e.fb : e.bb) == SENT;
+        return one ? (e.vf ? 0 : 1) : 2 + 4 * e.grp + std::max(e.vf, e.vb);
+    };
+    std::vector<int> ord64(t.nD), pos64(t.nD);
+    for (int j = 0; j < t.nD; ++j) ord64[j] = j;
+    std::stable_sort(ord64.begin(), ord64.end(), [&](int a, int b) { return kind64(ents[a]) < kind64(ents[b]); });
+    for (int j = 0; j < t.nD; ++j) {
+        const DEnt &e = ents[ord64[j]];
+        pos64[ord64[j]] = j;
+        if (kind64(e) <= 0) t.nD_F1++;
+        if (kind64(e) <= 1) t.nD_B1++;
+        t.d_pk64.push_back(make_int2(t.d_i0[ord64[j]], t.d_i1[ord64[j]]));
         t.d_ce.push_back(e.alpha1);
     }
     // gather lists: J_sk gathers nu_rs M_s D_rk over the reactions r (the
@@ -374,7 +399,7 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
         t.j_sk.push_back((s << 8) | k);
         t.j_sk32.push_back((s << 8) | k);
         for (const auto &tm : lists[idx]) {
-            t.j_d.push_back(tm.j);
+            t.j_d.push_back(pos64[tm.j]);
             t.j_c.push_back(tm.c);
             for (int part : pow2_parts(tm.nu)) {
                 t.j_d32.push_back(tm.j);
@@ -406,12 +431,30 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
         t.sp_item_ptr[s + 1] = (int)t.it_ptr.size() - 1;
     }
     t.n_items = (int)t.it_ptr.size() - 1;
-    // 2^(j/256), from the exponential of the exact arguments in long double
+    // the items run longest first, so that the last pass is a short one
+    // (sums are stored by item number)
+    {
+        std::vector<int> by_len(t.n_items), ptr{0}, r2, nu2;
+        for (int i = 0; i < t.n_items; ++i) by_len[i] = i;
+        std::stable_sort(by_len.begin(), by_len.end(), [&](int a, int b) {
+            return t.it_ptr[a + 1] - t.it_ptr[a] > t.it_ptr[b + 1] - t.it_ptr[b];
+        });
+        for (int i : by_len) {
+            for (int e = t.it_ptr[i]; e < t.it_ptr[i + 1]; ++e) {
+                r2.push_back(t.sp_r[e]);
+                nu2.push_back(t.sp_nui[e]);
+            }
+            ptr.push_back((int)r2.size());
+        }
+        t.it_id = by_len;
+        t.it_ptr.swap(ptr);
+        t.sp_r.swap(r2);
+        t.sp_nui.swap(nu2);
+    }
     // reciprocals for the elimination's small divisions (numerators below 64)
     t.div16.assign(67, 0u);
     for (int c = 1; c <= 66; ++c) t.div16[c] = (65536u + c - 1) / c;
-    t.exp_tab.resize(kExpTab);
-    for (int j = 0; j < kExpTab; ++j) t.exp_tab[j] = (double)std::exp2l((long double)j / kExpTab);
+    fill_exp_table(t.exp_tab);
     fill_log_table(t.log_tab);
     // FP32 copies for the mixed-precision Jacobian
     t.rxn_df.assign((size_t)nr * kRxnDStride, 0.0f);
@@ -531,7 +574,7 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
         }
         L.j_w.assign(std::max(nw32, 1), 0u);
         for (size_t e = 0; e < pos.size(); ++e) L.j_w[pos[e]] = t.j_w[e];
-        const int ni = interleave(t.n_items, t.it_ptr, G, L.it_meta, pos, 0, nullptr);
+        const int ni = interleave(t.n_items, t.it_ptr, G, L.it_meta, pos, 16, &t.it_id);
         L.sp_w.assign(std::max(ni, 1), 0u);
         for (size_t e = 0; e < pos.size(); ++e) {
             L.sp_w[pos[e]] = t.sp_w[e];
@@ -556,6 +599,7 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
     auto pad_f = [](std::vector<float> &v) { if (v.empty()) v.push_back(0.0f); };
     pad_f(t.rxn_df); pad_f(t.d_cef);
     if (t.d_pk.empty()) t.d_pk.push_back(make_int2(0, 0));
+    if (t.d_pk64.empty()) t.d_pk64.push_back(make_int2(0, 0));
     auto pad_u = [](std::vector<unsigned> &v) { if (v.empty()) v.push_back(0u); };
     pad_u(t.j_w); pad_u(t.sp_w);
     auto pad_i = [](std::vector<int> &v) { if (v.empty()) v.push_back(0); };
@@ -598,7 +642,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
         i_lay[li][4] = addv(L.it_meta);
         i_lay[li][5] = addv(L.sp_w);
     }
-    const size_t i_dce = addv(t.d_ce);
+    const size_t i_dce = addv(t.d_ce), i_dpk64 = addv(t.d_pk64);
     cudaError_t e = cudaMalloc(&h->dev_tables, total);
     if (e != cudaSuccess) return fail(CHEM_E_OOM, "device tables (%zu bytes): %s", total, cudaGetErrorString(e));
     h->dev_tables_bytes = total;
@@ -614,9 +658,8 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
     m.nr = nr;
     m.ntb = t.ntb;
     m.nD = t.nD;
-    m.nD_F = t.nD_F;
-    m.nD_B = t.nD_B;
-    m.nD_FB = t.nD_FB;
+    m.nD_F1 = t.nD_F1;
+    m.nD_B1 = t.nD_B1;
     m.nJ = t.nJ;
     m.nJ_nz = t.nJ_nz;
     m.n_items = t.n_items;
@@ -633,6 +676,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
     m.d_pk = (const int2 *)at(i_dpk);
     (void)i_gap;
     m.d_ce = (const double *)at(i_dce);
+    m.d_pk64 = (const int2 *)at(i_dpk64);
     for (int li = 0; li < kLayouts; ++li) {
         GatherLayout &g = m.gl[li];
         g.j_meta = (const int2 *)at(i_lay[li][0]);

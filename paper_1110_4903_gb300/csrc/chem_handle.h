@@ -71,5 +71,6 @@ int launch_cfg(Handle *h, const chem_advance_args *a, int prec, const LaunchCfg 
 unsigned long long *next_counter(Handle *h);
 StepOptions step_options(const Handle *h, int prec);
 void fill_log_table(std::vector<double> &tab);
+void fill_exp_table(std::vector<double> &tab);
 void destroy_serving(Handle *h);
 }  // namespace chem

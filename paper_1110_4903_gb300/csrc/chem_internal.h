@@ -67,13 +67,21 @@ constexpr int kMaxBlockThreads = 320;
 
 // Entries of the exp table (2^(j/kExpTab)).
 constexpr int kExpTab = 256;
+// FP64 constants that follow the exp table (the kernels take them as register
+// operands): 1, -0; 256/ln2, 1.5 * 2^52, -ln2/256 in two parts, 1/24, 1/6,
+// 1/2, 1 (the exponential); -1/6, 1/5, -1/4, 1/3, -1/2, ln 2 (the logarithm).
+constexpr int kConstOne = kExpTab, kConstExp = kExpTab + 2, kConstLog = kExpTab + 10;
+constexpr int kExpTabSize = kExpTab + 16;
 // Intervals of the log table: kLogTab + 1 entries {1/F, ln F}, F = 1 + j/kLogTab.
 constexpr int kLogTab = 128;
 
 // D entries: one per (reaction r, species k) pair whose concentration the
 // progress rate Q_r depends on, holding dQ_r/drho_k without the all-ones
-// third-body part.  They are sorted into four groups so each group is one
-// uniform loop: reactant-only, product-only, both sides, efficiency-only.
+// third-body part.  They are sorted into four groups: reactant-only,
+// product-only, both sides, efficiency-only.  The FP64 kernel keeps them in an
+// order of its own (d_pk64): [0, F1) reactant-only of order 1 with at most one
+// remaining factor, [F1, B1) the same for products, then the others, by
+// group and order.
 //   d_pk = {r | nu'_rk << 16 | nu''_rk << 20,
 //           fa | fb << 8 | ba << 16 | bb << 24  (the remaining factors of
 //                d(prod c)/dc_k on each side, sentinel ns if none)}
@@ -95,7 +103,7 @@ constexpr int kLogTab = 128;
 //                   (float)nu_rs (FP32 kernel: the row's M_s multiplies the
 //                   sum; terms ordered across the lanes of a pass for
 //                   distinct shared-memory banks)
-//   it_meta[i] = {first word of item i, entries}
+//   it_meta[i] = {first word, item number | entries << 16}, longest item first
 //   sp_w       = r (bits 0..19) | the sign and exponent bits of (double)nu_rs
 // (nu_rs a signed power of two in the words: any other nu_rs is split into
 // one term per binary digit)
@@ -116,7 +124,7 @@ __host__ __device__ constexpr int layout_index(int G) {
 struct DeviceMech {
     int ns, nr;
     int ntb;                    // third-body reactions: the first ntb (internal order)
-    int nD, nD_F, nD_B, nD_FB;  // group ends: [0,F) [F,B) [B,FB) [FB,nD)
+    int nD, nD_F1, nD_B1;       // D entries; ends of the FP64 order's first groups
     int nJ;                     // Jacobian entries gathered: ns*ns (species rows and columns)
     int nJ_nz;                  //   of which the first nJ_nz have reaction terms (longest list first)
     int n_items;                // species-gather work items
@@ -130,14 +138,15 @@ struct DeviceMech {
     const int *eff_ptr;         // [nr+1] CSR of efficiency corrections of +M reactions
     const int *eff_sp;          //        species
     const double *eff_c;        //        alpha - 1
-    const int2 *d_pk;           // [nD]
+    const int2 *d_pk;           // [nD] (FP32 kernel)
+    const int2 *d_pk64;         // [nD] (FP64 kernel's order)
     const double *d_ce;         // [nD] alpha - 1 (FP64 kernel)
     // Jacobian entries (species rows and columns), longest gather list
     // first, and the species lists (reactions with nu_rs != 0) cut into
     // items of at most kChunk entries; per-G layouts above
     GatherLayout gl[kLayouts];
     const int *sp_item_ptr;     // [ns+1] work items of each species
-    const double *exp_tab;      // [kExpTab] 2^(j/kExpTab)
+    const double *exp_tab;      // [kExpTab] 2^(j/kExpTab), then the constants above
     const double2 *log_tab;     // [kLogTab + 1] {1/F, ln F}, F = 1 + j/kLogTab
     const unsigned *div16;      // [67] ceil(2^16 / c): x / c = (x div16[c]) >> 16 for x < 64
     // FP32 copies for the mixed-precision Jacobian

@@ -66,6 +66,32 @@ enum SlotAction : int {
     kEmitCell = 3
 };
 
+// The FP64 pipe takes a warp's fused multiply-add with three register
+// operands every 16 cycles, but an addition, a multiplication or anything
+// with a constant operand only every 19 (measured, 4 to 20 warps on an SM).
+// So sums and products are written as fused multiply-adds with a 1 and a -0
+// in registers (the same results, signed zeros included), and constants come
+// from a table in global memory.  The loads are volatile: the compiler must
+// not see the values, nor keep all of them in registers.
+struct Fp64Ops {
+    double one, nz;   // 1 and -0
+    __device__ __forceinline__ double add(double a, double b) const { return __fma_rn(a, one, b); }
+    __device__ __forceinline__ double sub(double a, double b) const { return __fma_rn(-b, one, a); }
+    __device__ __forceinline__ double mul(double a, double b) const { return __fma_rn(a, b, nz); }
+};
+__device__ __forceinline__ double2 ld_const2(const double *p) {
+    double2 v;
+    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];"
+                 : "=d"(v.x), "=d"(v.y)
+                 : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+// (tab: the exp table, which the constants follow)
+__device__ __forceinline__ Fp64Ops fp64_ops(const double *tab) {
+    const double2 v = ld_const2(tab + kConstOne);
+    return Fp64Ops{v.x, v.y};
+}
+
 template <int G>
 struct Grp {
     template <typename V>
@@ -74,10 +100,9 @@ struct Grp {
         for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
         return v;
     }
-    template <typename V>
-    __device__ __forceinline__ static V max(V v) {
+    __device__ __forceinline__ static double sum(double v, const Fp64Ops &op) {
 #pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
+        for (int o = G / 2; o > 0; o >>= 1) v = op.add(v, __shfl_xor_sync(kFull, v, o));
         return v;
     }
     __device__ __forceinline__ static int any(int v) {
@@ -206,19 +231,19 @@ using PivotKey = decltype(abs_key(JT(0)));
 // Reciprocal: the hardware approximation r refined with its residual
 // e = 1 - a r as r (1 + e + e^2), whose error is e^3 (the approximation is
 // good to about 2^-23, so below FP64 rounding): three FP64 operations.
-__device__ __forceinline__ double frcp(double a) {
+__device__ __forceinline__ double frcp(double a, const Fp64Ops &op) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    const double e = fma(-a, r, 1.0);
+    const double e = fma(-a, r, op.one);
     return fma(r, fma(e, e, e), r);
 }
 // One Newton step only (relative error about 1e-14): for reciprocals that
 // scale a convergence ratio or the temperature recovery's Newton step, never
 // a rate, an energy or the elimination.
-__device__ __forceinline__ double frcp1(double a) {
+__device__ __forceinline__ double frcp1(double a, const Fp64Ops &op) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    const double e = fma(-a, r, 1.0);
+    const double e = fma(-a, r, op.one);
     return fma(r, e, r);
 }
 // FP32 reciprocal of the pivot: the hardware approximation (within an ulp or
@@ -261,24 +286,32 @@ __device__ __forceinline__ double small_pos_int_to_double(int v) {
 // exp by the table-driven reduction of P. T. P. Tang, ACM TOMS 15(2), 1989:
 // x = (256 k + j) ln2/256 + r with |r| <= ln2/512, exp(x) = 2^k 2^(j/256) e^r,
 // 2^(j/256) from a 256-entry table and e^r - 1 by its degree-4 Taylor
-// polynomial (truncation below 4e-17 on that interval): nine FP64
-// operations.  |x| >= 512, infinities and NaN (decided on the exponent bits,
-// no FP64 compare) fall back to the library exp.
-__device__ __forceinline__ double fexp(double x, const double *tab) {
+// polynomial (truncation below 4e-17 on that interval): eight FP64
+// operations (the integer n = 256 k + j becomes a double on the integer
+// pipe).  exp_reduced: y 2^(n >> 8) = exp(x) for |x| < 2^22, n below 2^31.
+__device__ __forceinline__ double exp_reduced(double x, const double *tab, const Fp64Ops &op, int &n,
+                                              bool n_small) {
+    const double2 c0 = ld_const2(tab + kConstExp), c1 = ld_const2(tab + kConstExp + 2),
+                  c2 = ld_const2(tab + kConstExp + 4), c3 = ld_const2(tab + kConstExp + 6);
+    const double t = fma(x, c0.x, c0.y);   // x * 256/ln2 + 1.5 * 2^52: rounded to an integer
+    n = (int)(unsigned)__double_as_longlong(t);
+    const double nd = n_small ? f2d_alu(small_int_to_float(n)) : op.sub(t, c0.y);
+    double r = fma(nd, c1.x, x);           // - n ln2/256, high 36 bits
+    r = fma(nd, c1.y, r);                  // low part
+    double p = fma(r, c2.x, c2.y);
+    p = fma(r, p, c3.x);
+    p = fma(r, p, op.one);
+    p = op.mul(p, r);                      // e^r - 1
+    const double s = __ldg(tab + (n & (kExpTab - 1)));
+    return fma(s, p, s);
+}
+// |x| >= 512, infinities and NaN (decided on the exponent bits, no FP64
+// compare) fall back to the library exp.
+__device__ __forceinline__ double fexp(double x, const double *tab, const Fp64Ops &op) {
     const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32);
     if (((hi >> 20) & 0x7ffu) > 0x407u) return exp_outside(x);
-    const double kShift = 6755399441055744.0;               // 1.5 * 2^52
-    const double t = fma(x, 369.3299304675746, kShift);     // x * 256/ln2, rounded
-    const int n = (int)(unsigned)__double_as_longlong(t);
-    const double nd = t - kShift;
-    double r = fma(nd, -0x1.62e42fefa0000p-9, x);            // ln2/256, high 36 bits
-    r = fma(nd, -0x1.cf79abc9e3b3ap-48, r);                  // ln2/256, low part
-    double p = fma(r, 1.0 / 24.0, 1.0 / 6.0);
-    p = fma(r, p, 0.5);
-    p = fma(r, p, 1.0);
-    p *= r;                                                  // e^r - 1
-    const double s = __ldg(tab + (n & (kExpTab - 1)));
-    const double y = fma(s, p, s);
+    int n;
+    const double y = exp_reduced(x, tab, op, n, true);   // |n| < 2^18
     const long long k = (long long)(n >> 8);
     return __longlong_as_double(__double_as_longlong(y) + (k << 52));
 }
@@ -289,7 +322,7 @@ __device__ __forceinline__ double fexp(double x, const double *tab) {
 // any |x| < 2^22 (the products with ln2/256 are fused, and the table index
 // fits an int); beyond that (and for infinities) k saturates at +-2^24 with
 // y = 1, and a NaN x gives a NaN y.
-__device__ __forceinline__ void split_exp(double x, const double *tab, double &y, int &k) {
+__device__ __forceinline__ void split_exp(double x, const double *tab, const Fp64Ops &op, double &y, int &k) {
     const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32);
     const unsigned ex = (hi >> 20) & 0x7ffu;
     if (ex >= 0x415u) {
@@ -298,18 +331,8 @@ __device__ __forceinline__ void split_exp(double x, const double *tab, double &y
         k = (hi >> 31) ? -(1 << 24) : (1 << 24);
         return;
     }
-    const double kShift = 6755399441055744.0;               // 1.5 * 2^52
-    const double t = fma(x, 369.3299304675746, kShift);     // x * 256/ln2, rounded
-    const int n = (int)(unsigned)__double_as_longlong(t);
-    const double nd = t - kShift;
-    double r = fma(nd, -0x1.62e42fefa0000p-9, x);
-    r = fma(nd, -0x1.cf79abc9e3b3ap-48, r);
-    double p = fma(r, 1.0 / 24.0, 1.0 / 6.0);
-    p = fma(r, p, 0.5);
-    p = fma(r, p, 1.0);
-    p *= r;
-    const double s = __ldg(tab + (n & (kExpTab - 1)));
-    y = fma(s, p, s);
+    int n;
+    y = exp_reduced(x, tab, op, n, false);
     k = n >> 8;
 }
 // v 2^k on the exponent bits for a normal v; zero, subnormal, infinite and
@@ -335,28 +358,29 @@ __device__ __forceinline__ double scale_pow2(double v, int k) {
 // the result can be small next to k ln2 + ln F, and the table's rounding
 // then leaves an absolute error near 1e-16.  The kernels take it of T in
 // [200, 6000] K.)
-__device__ __forceinline__ double flog(double x, const double2 *tab) {
+__device__ __forceinline__ double flog(double x, const double2 *tab, const double *exp_tab, const Fp64Ops &op) {
     const long long b = __double_as_longlong(x);
     const int k = (int)(b >> 52) - 1023;
     const double y = __longlong_as_double((b & 0x000fffffffffffffLL) | 0x3ff0000000000000LL);
     const int j = (int)((b >> 45) & 0x7f) + (int)((b >> 44) & 1);
     const double F = __longlong_as_double(0x3ff0000000000000LL + ((long long)j << 45));
     const double2 t = __ldg(tab + j);
-    const double u = (y - F) * t.x;
-    double p = fma(u, -1.0 / 6.0, 0.2);
-    p = fma(u, p, -0.25);
-    p = fma(u, p, 1.0 / 3.0);
-    p = fma(u, p, -0.5);
-    p = fma(u, p, 1.0);
-    // k as a double: added to the bit pattern of 1.5 * 2^52, whose ulp is 1
-    const double kd = __longlong_as_double(0x4338000000000000LL + k) - 6755399441055744.0;
-    return fma(u, p, fma(kd, 0.6931471805599453, t.y));
+    const double2 c0 = ld_const2(exp_tab + kConstLog), c1 = ld_const2(exp_tab + kConstLog + 2),
+                  c2 = ld_const2(exp_tab + kConstLog + 4);
+    const double u = op.mul(op.sub(y, F), t.x);
+    double p = fma(u, c0.x, c0.y);   // -1/6, 1/5
+    p = fma(u, p, c1.x);             // -1/4
+    p = fma(u, p, c1.y);             // 1/3
+    p = fma(u, p, c2.x);             // -1/2
+    p = fma(u, p, op.one);
+    const double kd = f2d_alu(small_int_to_float(k));
+    return fma(u, p, fma(kd, c2.y, t.y));   // ln 2
 }
 
 // NASA-7 entropy from the thermo coefficients of one species and range
 // (layout in chem_internal.h)
-__device__ __forceinline__ double nasa_s(const CoefRow<double> &th, double T, double lnT) {
-    return th[0] * lnT + T * (th[1] + T * (th[10] + T * (th[11] + T * th[12]))) + th[13];
+__device__ __forceinline__ double nasa_s(const CoefRow<double> &th, double T, double lnT, const Fp64Ops &op) {
+    return op.add(fma(th[0], lnT, op.mul(T, fma(T, fma(T, fma(T, th[12], th[11]), th[10]), th[1]))), th[13]);
 }
 // range of species s at T (1: T > T_mid, the high range)
 __device__ __forceinline__ int thermo_range(const DeviceMech &m, int s, long long Tbits) {
@@ -371,9 +395,10 @@ __device__ __forceinline__ int thermo_range(const DeviceMech &m, int s, long lon
 //   species, no 1/T); with F32 the derivative sum c_v is formed in FP32, which
 //   changes the Newton steps by a relative 1e-7 and not the root.
 template <int G, bool F32>
-__device__ __forceinline__ void recover_T(const DeviceMech &m, const double *x, int sl, bool need,
+__device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab, const double *x, int sl, bool need,
                                           double guess, double &T_out, bool &ok) {
     const int ns = m.ns;
+    const Fp64Ops op = fp64_ops(tab);
     double lo = kTlo, hi = kThi, T = guess;
     if (!(bits_gt(T, lo) && bits_lt(T, hi))) T = 1500.0;
     bool done = !need;
@@ -401,14 +426,14 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *x, 
                 fp = fma(x[s], cv, fp);
             }
         }
-        f = Grp<G>::sum(f) - e;
+        f = op.sub(Grp<G>::sum(f, op), e);
         double rfp;
         if (F32) {
             fpf = Grp<G>::sum(fpf);
             rfp = f2d_alu(__frcp_rn(fpf));
         } else {
-            fp = Grp<G>::sum(fp);
-            rfp = frcp1(fp);
+            fp = Grp<G>::sum(fp, op);
+            rfp = frcp1(fp, op);
         }
         if (!done) {
             const long long fb = __double_as_longlong(f);
@@ -420,9 +445,9 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *x, 
                     hi = T;
                 else
                     lo = T;
-                double Tn = T - f * rfp;
+                double Tn = fma(-f, rfp, T);
                 if (!(bits_gt(Tn, lo) && bits_lt(Tn, hi))) Tn = 0.5 * (lo + hi);
-                const double dT = Tn - T;
+                const double dT = op.sub(Tn, T);
                 T = Tn;
                 // (comparisons of non-negative doubles on their bit patterns)
                 if (!bits_gt(fabs(dT), kTtol * T)) {
@@ -732,9 +757,23 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     // the 16-byte accesses of its elimination; the right-hand side is column N)
     const int N = ns, ldA = N + 1, ldc = (N + 3) & ~3;
     auto ix = [&](int i, int k) -> int { return f32 ? k * ldc + i : i * ldA + k; };
-    const double invT = frcp(T);
-    const double lnT = flog(T, m.log_tab);   // T in [200, 6000] K: normal
-    const double lnPaRT = kLnPaOverR - lnT;
+    const Fp64Ops op = fp64_ops(tab);
+    // sums and products in the Jacobian type
+    auto jadd = [&](JT a, JT b) -> JT {
+        if constexpr (f32)
+            return a + b;
+        else
+            return op.add(a, b);
+    };
+    auto jmul = [&](JT a, JT b) -> JT {
+        if constexpr (f32)
+            return a * b;
+        else
+            return op.mul(a, b);
+    };
+    const double invT = frcp(T, op);
+    const double lnT = flog(T, m.log_tab, tab, op);   // T in [200, 6000] K: normal
+    const double lnPaRT = op.sub(kLnPaOverR, lnT);
 
     // 1. concentrations and thermodynamics (species); the heat capacity only
     //    feeds dT/drho, dT/de and the next temperature guess, so the FP32
@@ -747,21 +786,21 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     for (int s = sl; s < ns; s += G) {
         const double *spr = m.sp + s * kSpStride;
         const double xs = sm.x[s];
-        const double ci = xs * __ldg(spr + 1);
+        const double ci = op.mul(xs, __ldg(spr + 1));
         sm.c[s] = ci;
-        ctot += ci;
+        ctot = op.add(ctot, ci);
         const int rg = thermo_range(m, s, Tb);
         const auto th = coef_row(m.thermo, ns, s, rg);
-        const double hRT = th[0] + T * (th[5] + T * (th[6] + T * (th[7] + T * th[8]))) + th[9] * invT;
-        const double sR = nasa_s(th, T, lnT);
+        const double hRT = fma(th[9], invT, fma(T, fma(T, fma(T, fma(T, th[8], th[7]), th[6]), th[5]), th[0]));
+        const double sR = nasa_s(th, T, lnT, op);
         const double RM = __ldg(spr + 2);
         // exp(g_s/RT - ln(P_a/RT)) split into mantissa and power of two,
         // for the equilibrium constants (phase 2)
         double ey;
         int eK;
-        split_exp(hRT - sR - lnPaRT, tab, ey, eK);
+        split_exp(op.sub(op.sub(hRT, sR), lnPaRT), tab, op, ey, eK);
         sm.em[s] = ey;
-        sm.emi[s] = frcp(ey);
+        sm.emi[s] = frcp(ey, op);
         sm.ek[s] = eK;
         if (f32) {
             // the species energy with its formation part, e_s = (R/M) T (h/RT
@@ -775,7 +814,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             sm.cJ[s] = to_jt<JT>(ci);
             sm.hJ[s] = hJs;
         } else {
-            const double es = RM * T * (hRT - 1.0) - __ldg(spr + 3);
+            const double es = fma(op.mul(RM, T), op.sub(hRT, op.one), -__ldg(spr + 3));
             const auto c = coef_row(m.tpoly, ns, s, rg);
             const double cv = fma(fma(fma(fma(c[10], T, c[9]), T, c[8]), T, c[7]), T, c[6]);
             rhocv = fma(xs, cv, rhocv);
@@ -796,7 +835,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             sm.hRT[ns] = 0.0;
         }
     }
-    ctot = Grp<G>::sum(ctot);
+    ctot = Grp<G>::sum(ctot, op);
     double dTde;
     float dTdef = 0.f;
     if (f32) {
@@ -805,10 +844,10 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         dTde = f2d_alu(dTdef);
         // dT/drho_k = -e_k^sens dT/de is formed where the Jacobian needs it
     } else {
-        rhocv = Grp<G>::sum(rhocv);
-        dTde = frcp(rhocv);
+        rhocv = Grp<G>::sum(rhocv, op);
+        dTde = frcp(rhocv, op);
 #pragma unroll 1
-        for (int s = sl; s < ns; s += G) sm.dTdr[s] = (JT)(-(sm.es[s] + __ldg(m.sp + s * kSpStride + 3)) * dTde);
+        for (int s = sl; s < ns; s += G) sm.dTdr[s] = (JT)op.mul(-op.add(sm.es[s], __ldg(m.sp + s * kSpStride + 3)), dTde);
     }
     __syncwarp();
 
@@ -842,10 +881,14 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         // mechanism has at most two per side); the vote makes the branch
         // uniform, so the skipped FP64 products cost no pipe slot
         const bool s3 = __any_sync(__activemask(), (a2 != ns) | (b2 != ns));
-        double Pf = sm.c[a0] * sm.c[a1];
-        double Pb = sm.c[b0] * sm.c[b1];
-        const double lnkf = lnA + beta * lnT - EaR * invT;
-        const double kf = fexp(lnkf, tab);
+        double Pf = op.mul(sm.c[a0], sm.c[a1]);
+        double Pb = op.mul(sm.c[b0], sm.c[b1]);
+        // (the FP64 path rounds E/RT and the forward rate by themselves: its
+        // temperature derivatives use them too)
+        const double EaRT = f32 ? 0.0 : op.mul(EaR, invT);
+        const double lnAT = fma(beta, lnT, lnA);
+        const double lnkf = f32 ? fma(-EaR, invT, lnAT) : op.sub(lnAT, EaRT);
+        const double kf = fexp(lnkf, tab, op);
         // K_b = K_f / K_c with 1/K_c = (RT/P_a)^dnu exp(dG/RT) (Eq. 24) as
         // the product over the factor slots of the species' exp(g/RT) (RT/P_a)
         // (products) and their inverses (reactants), the sentinel giving 1:
@@ -854,24 +897,26 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         int K2 = (sm.ek[b0] + sm.ek[b1]) - (sm.ek[a0] + sm.ek[a1]);
         double Pm;
         if (s3) {
-            Pf *= sm.c[a2];
-            Pb *= sm.c[b2];
+            Pf = op.mul(Pf, sm.c[a2]);
+            Pb = op.mul(Pb, sm.c[b2]);
             K2 = (sm.ek[b0] + sm.ek[b1] + sm.ek[b2]) - (sm.ek[a0] + sm.ek[a1] + sm.ek[a2]);
-            Pm = ((sm.em[b0] * sm.em[b1]) * sm.em[b2]) * ((sm.emi[a0] * sm.emi[a1]) * sm.emi[a2]);
+            Pm = op.mul(op.mul(op.mul(sm.em[b0], sm.em[b1]), sm.em[b2]),
+                        op.mul(op.mul(sm.emi[a0], sm.emi[a1]), sm.emi[a2]));
         } else {
-            Pm = (sm.em[b0] * sm.em[b1]) * (sm.emi[a0] * sm.emi[a1]);
+            Pm = op.mul(op.mul(sm.em[b0], sm.em[b1]), op.mul(sm.emi[a0], sm.emi[a1]));
         }
-        const double kb = scale_pow2(kf * Pm, K2);
+        const double kb = scale_pow2(op.mul(kf, Pm), K2);
         double CM = 1.0;
         const bool tb = (fr >> 24) & 1;
         if (tb) {
             CM = ctot;
             const int e0 = __ldg(m.eff_ptr + r), e1 = __ldg(m.eff_ptr + r + 1);
 #pragma unroll 1
-            for (int e = e0; e < e1; ++e) CM += __ldg(m.eff_c + e) * sm.c[__ldg(m.eff_sp + e)];
+            for (int e = e0; e < e1; ++e) CM = fma(__ldg(m.eff_c + e), sm.c[__ldg(m.eff_sp + e)], CM);
         }
-        const double fwd = kf * Pf, rev = kb * Pb, q = fwd - rev;
-        sm.Q[r] = CM * q;   // in the D region until phase 4
+        const double rev = op.mul(kb, Pb), fwd = f32 ? 0.0 : op.mul(kf, Pf);
+        const double q = f32 ? fma(kf, Pf, -rev) : op.sub(fwd, rev);
+        sm.Q[r] = op.mul(CM, q);   // in the D region until phase 4
         if (f32) {
             // Jacobian-only quantities in FP32 from FP32 copies
             const float *rf = m.rxn_df + (size_t)r * kRxnDStride;
@@ -895,14 +940,15 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             }
             sm.dQdT[r] = A1v * PfJ * dlnkf - A2v * PbJ * (dlnkf - dlnKc);
         } else {
-            const double sh = s3 ? (sm.hRT[b0] + sm.hRT[b1] + sm.hRT[b2]) - (sm.hRT[a0] + sm.hRT[a1] + sm.hRT[a2])
-                                 : (sm.hRT[b0] + sm.hRT[b1]) - (sm.hRT[a0] + sm.hRT[a1]);
+            const double hb = op.add(sm.hRT[b0], sm.hRT[b1]), ha = op.add(sm.hRT[a0], sm.hRT[a1]);
+            const double sh = s3 ? op.sub(op.add(hb, sm.hRT[b2]), op.add(ha, sm.hRT[a2])) : op.sub(hb, ha);
             if (r < m.ntb) sm.qtb[r] = (JT)q;
-            sm.A1[r] = (JT)(CM * kf);
-            sm.A2[r] = (JT)(CM * kb);
-            const double dlnkf = fma(EaR * invT, invT, beta * invT);
-            const double dlnKc = (sh - dnu) * invT;
-            sm.dQdT[r] = (JT)(CM * (fwd * dlnkf - rev * (dlnkf - dlnKc)));
+            sm.A1[r] = (JT)op.mul(CM, kf);
+            sm.A2[r] = (JT)op.mul(CM, kb);
+            const double dlnkf = fma(EaRT, invT, op.mul(beta, invT));
+            // (d ln K_b/dT = d ln K_f/dT - (sh - dnu) / T)
+            const double dlnkb = fma(-op.sub(sh, dnu), invT, dlnkf);
+            sm.dQdT[r] = (JT)op.mul(CM, fma(fwd, dlnkf, -op.mul(rev, dlnkb)));
         }
     }
     __syncwarp();
@@ -928,18 +974,18 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     };
     static_assert(kChunk == 8, "an item is two groups of four terms");
     int2 im = item_at(sl);
-    uint4 iwords = item_words(im.x, im.y);
+    uint4 iwords = item_words(im.x, im.y >> 16);
 #pragma unroll 1
     for (int it = sl; it < m.n_items; it += G) {
-        const int e1 = im.x + 4 * G;
-        int rem = im.y;
+        const int e1 = im.x + 4 * G, id = im.y & 0xffff;
+        int rem = im.y >> 16;
         im = item_at(it + G);
         double sq = 0.0;
         JT sdq = 0, squ = 0;
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
             const uint4 wc = iwords;
-            iwords = half == 0 ? item_words(e1, rem - 4) : item_words(im.x, im.y);
+            iwords = half == 0 ? item_words(e1, rem - 4) : item_words(im.x, im.y >> 16);
             const unsigned wv[4] = {wc.x, wc.y, wc.z, wc.w};
             double Qv[4];
             JT dq[4], qt[4];
@@ -964,8 +1010,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             rem -= 4;
         }
         constexpr int iw = (int)(item_bytes((int)sizeof(JT)) / 8);   // doubles per item
-        sm.part[iw * it] = sq;
-        JT *pj = reinterpret_cast<JT *>(sm.part + iw * it + 1);
+        sm.part[iw * id] = sq;
+        JT *pj = reinterpret_cast<JT *>(sm.part + iw * id + 1);
         pj[0] = sdq;
         pj[1] = squ;
     }
@@ -979,19 +1025,19 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         constexpr int iw = (int)(item_bytes((int)sizeof(JT)) / 8);
 #pragma unroll 1
         for (int it = i0; it < i1; ++it) {
-            sq += sm.part[iw * it];
+            sq = op.add(sq, sm.part[iw * it]);
             const JT *pj = reinterpret_cast<const JT *>(sm.part + iw * it + 1);
-            sdq += pj[0];
-            squ += pj[1];
+            sdq = jadd(sdq, pj[0]);
+            squ = jadd(squ, pj[1]);
         }
         const double M = __ldg(m.sp + s * kSpStride);
         const double ef = __ldg(m.sp + s * kSpStride + 3);
         const JT MJ = f32 ? (JT)__ldg(m.spf + s * kSpStride) : (JT)M;
-        const double wds = M * sq;
+        const double wds = op.mul(M, sq);
         // right-hand side -F_s = -(x_s - x0_s - h wdot_s), FP64 until stored
-        const double dx = sm.x[s] - sm.x0[s];
-        sm.rhs[s] = to_jt<JT>(-(dx - h * wds));
-        const JT ws = MJ * sdq, us = MJ * squ;
+        const double dx = op.sub(sm.x[s], sm.x0[s]);
+        sm.rhs[s] = to_jt<JT>(-fma(-h, wds, dx));
+        const JT ws = jmul(MJ, sdq), us = jmul(MJ, squ);
         sm.w[s] = ws;
         sm.u[s] = us;
         dEt = fma(ef, dx, dEt);
@@ -999,7 +1045,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     // the total-energy residual R_E = F_e + sum_s e_f,s F_s = (x_e - x0_e) +
     // sum_s e_f,s (x_s - x0_s), in which the sources cancel (Omega_e =
     // -sum_s e_f,s wdot_s); it replaces the energy equation (phase 5)
-    const double RE = Grp<G>::sum(dEt) + (sm.x[ns] - sm.x0[ns]);
+    const double RE = op.add(Grp<G>::sum(dEt, op), op.sub(sm.x[ns], sm.x0[ns]));
     __syncwarp();
 
     // 4. D entries: d Q_r / d rho_k without the all-ones third-body part,
@@ -1036,19 +1082,26 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         // the FP64 D entries are M_k dQ_r/drho_k as well: integer orders from
         // the descriptor (exact doubles by integer operations), alpha - 1
         // from an 8-byte table, and the gather applies the 1/M_k
-        const int2 pk = __ldg(m.d_pk + j);
+        // (in an order of their own: first those with order 1 and one
+        // remaining factor, one multiplication instead of three)
+        const int2 pk = __ldg(m.d_pk64 + j);
         const int r = pk.x & 0xffff, vf = (pk.x >> 16) & 15, vb = (pk.x >> 20) & 15, i1 = pk.y;
         const int fa = i1 & 0xff, fb = (i1 >> 8) & 0xff, ba = (i1 >> 16) & 0xff, bb = (i1 >> 24) & 0xff;
+        // (one side's factors, selected without a branch; the reactant side
+        // where a species is on both)
         double dd;
-        if (j < m.nD_F) {
-            dd = small_pos_int_to_double(vf) * sm.A1[r] * (sm.c[fa] * sm.c[fb]);
-        } else if (j < m.nD_B) {
-            dd = -(small_pos_int_to_double(vb) * sm.A2[r] * (sm.c[ba] * sm.c[bb]));
-        } else if (j < m.nD_FB) {
-            dd = small_pos_int_to_double(vf) * sm.A1[r] * (sm.c[fa] * sm.c[fb]) -
-                 small_pos_int_to_double(vb) * sm.A2[r] * (sm.c[ba] * sm.c[bb]);
+        if (j < m.nD_B1) {
+            const bool f = j < m.nD_F1;
+            dd = op.mul(f ? sm.A1[r] : sm.A2[r], sm.c[f ? fa : ba]);
+            if (!f) dd = -dd;
         } else {
-            dd = 0.0;
+            const bool f = vf > 0;
+            const double v = small_pos_int_to_double(f ? vf : max(vb, 1));
+            const double A = op.mul(v, f ? sm.A1[r] : sm.A2[r]), cc = op.mul(sm.c[f ? fa : ba], sm.c[f ? fb : bb]);
+            dd = op.mul(A, cc);
+            if (!f) dd = vb > 0 ? -dd : 0.0;
+            if (f && vb > 0)
+                dd = fma(A, cc, -op.mul(op.mul(small_pos_int_to_double(vb), sm.A2[r]), op.mul(sm.c[ba], sm.c[bb])));
         }
         sm.D[j] = r < m.ntb ? (JT)fma(__ldg(m.d_ce + j), (double)sm.qtb[r], dd) : (JT)dd;
     }
@@ -1066,7 +1119,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     //    arithmetic, with one unknown fewer and no energy row to form
     const JT mh = to_jt<JT>(-h);
     {
-        const JT cRE = f32 ? mh * (JT)dTdef * d2f_rz(RE) : (JT)(-h * dTde * RE);
+        const JT cRE = f32 ? mh * (JT)dTdef * d2f_rz(RE) : (JT)op.mul(op.mul(-h, dTde), RE);
 #pragma unroll 1
         for (int i = sl; i < N; i += G) sm.A[ix(i, N)] = fma(sm.w[i], cRE, sm.rhs[i]);
     }
@@ -1196,7 +1249,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             mn = meta_at(p + 2 * G);
             tn = terms_at(me.x, me.y >> 16);
             const JT invMk = (JT)__ldg(m.sp + k * kSpStride + 1);
-            const JT J = sm.w[s] * sm.dTdr[k];
+            const JT J = jmul(sm.w[s], sm.dTdr[k]);
             JT ua = sm.u[s];
             if (len > 0) {
                 JT a0 = 0, a1 = 0;
@@ -1220,15 +1273,15 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
                     }
                     if (rem <= 0) break;
                 }
-                if (len >= 4) a0 += a1;
-                ua += a0;
+                if (len >= 4) a0 = jadd(a0, a1);
+                ua = jadd(ua, a0);
             }
             // (D entries scaled by M_k; the FP64 lists' coefficients are nu_rs M_s)
-            sm.A[ix(s, k)] = mh * fma(invMk, ua, J);
+            sm.A[ix(s, k)] = jmul(mh, fma(invMk, ua, J));
         }
         __syncwarp();
 #pragma unroll 1
-        for (int i = sl; i < N; i += G) sm.A[ix(i, i)] += (JT)1;
+        for (int i = sl; i < N; i += G) sm.A[ix(i, i)] = jadd(sm.A[ix(i, i)], (JT)op.one);
         __syncwarp();
     }
 
@@ -1270,10 +1323,14 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         // (the FP64 pivot takes the full-precision reciprocal: a 1e-14 error
         // in every multiplier reaches the trace species of ill-conditioned
         // cells at 1e-10)
-        const JT inv = frcp(sm.A[ix(j, j)]);
+        JT inv;
+        if constexpr (f32)
+            inv = frcp(sm.A[ix(j, j)]);
+        else
+            inv = frcp(sm.A[ix(j, j)], op);
         if (!f32) {
 #pragma unroll 1
-            for (int i = j + 1 + sl; i < N; i += G) sm.A[i * ldA + j] *= inv;
+            for (int i = j + 1 + sl; i < N; i += G) sm.A[i * ldA + j] = jmul(sm.A[i * ldA + j], inv);
             __syncwarp();
             if (sl == 0) sm.A[j * ldA + j] = inv;
         }
@@ -1313,7 +1370,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     // back substitution, U delta = y
 #pragma unroll 1
         for (int j = N - 1; j >= 0; --j) {
-            const JT dj = sm.A[ix(j, N)] * sm.A[ix(j, j)];
+            const JT dj = jmul(sm.A[ix(j, N)], sm.A[ix(j, j)]);
             __syncwarp();
             if (sl == 0) sm.A[ix(j, N)] = dj;
 #pragma unroll 1
@@ -1328,8 +1385,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     //    paths (they decide acceptance and the divergence abort) and their
     //    maximum is taken on the bit patterns; a zero scale counts a nonzero
     //    update as infinitely large.
-    auto ratio = [](double d, double den) -> double {
-        if (__double_as_longlong(den) > 0) return fabs(d) * frcp1(den);
+    auto ratio = [&](double d, double den) -> double {
+        if (__double_as_longlong(den) > 0) return op.mul(fabs(d), frcp1(den, op));
         return (__double_as_longlong(d) << 1) != 0 ? CUDART_INF : 0.0;
     };
     double nrm = 0.0, des = 0.0, se = 0.0;
@@ -1346,10 +1403,10 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             sef = fmaf(__ldg(m.spf + i * kSpStride + 3), df, sef);
         } else {
             d = (double)sm.A[ix(i, N)];
-            des -= sm.es[i] * d;
+            des = fma(-sm.es[i], d, des);
             se = fma(__ldg(m.sp + i * kSpStride + 3), d, se);
         }
-        const double xi = sm.x[i] + d;
+        const double xi = op.add(sm.x[i], d);
         sm.x[i] = xi;
         if (!finite_bits(xi)) nonfinite = 1;
         const double ri = ratio(d, fma(rtol, fabs(xi), atol_rho));
@@ -1357,9 +1414,9 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     }
     {
         // the eliminated energy unknown: de = -R_E - e_f . drho
-        const double de = -RE - (f32 ? f2d_alu(Grp<G>::sum(sef)) : Grp<G>::sum(se));
+        const double de = op.sub(-RE, f32 ? f2d_alu(Grp<G>::sum(sef)) : Grp<G>::sum(se, op));
         if (sl == 0) {
-            const double xe = sm.x[ns] + de;
+            const double xe = op.add(sm.x[ns], de);
             sm.x[ns] = xe;
             if (!finite_bits(xe)) nonfinite = 1;
             const double ri = ratio(de, fma(rtol, fabs(xe), atol_e));
@@ -1369,7 +1426,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             if (f32)
                 desf += d2f_rz(-RE);
             else
-                des += de;
+                des = op.add(des, de);
         }
     }
     nrm = Grp<G>::max_nonneg(nrm);
@@ -1377,11 +1434,11 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     if (f32)
         des = f2d_alu(Grp<G>::sum(desf));
     else
-        des = Grp<G>::sum(des);
+        des = Grp<G>::sum(des, op);
     __syncwarp();
     norm = nrm;
     bad = sing || nonfinite;
-    T_pred = T + des * dTde;
+    T_pred = fma(des, dTde, T);
 }
 
 // ---- request-server queue (ServeQueue in chem_internal.h) -----------------
@@ -1711,7 +1768,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
             if (!__any_sync(kFull, needT || act != kNoAction)) break;
             double Tr = T;
             bool ok = false;
-            recover_T<G, sizeof(JT) == 4>(m, sm.x, sl, needT, T, Tr, ok);
+            recover_T<G, sizeof(JT) == 4>(m, tab, sm.x, sl, needT, T, Tr, ok);
             int neg = 0;
 #pragma unroll 1
             for (int i = sl; i < ns; i += G)

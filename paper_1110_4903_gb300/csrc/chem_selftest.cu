@@ -18,9 +18,10 @@ __global__ void selftest_kernel(long long n, const double *x, const double *tab_
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double v = x[i];
-    y_exp[i] = fexp(v, tab);
+    const Fp64Ops op = fp64_ops(tab);
+    y_exp[i] = fexp(v, tab, op);
     y_exp_ref[i] = exp(v);
-    y_rcp[i] = frcp(v);
+    y_rcp[i] = frcp(v, op);
     y_rcp_ref[i] = 1.0 / v;
 }
 
@@ -30,18 +31,18 @@ __global__ void selftest_scaled_exp_kernel(long long n, const double *x, const d
     if (i >= n) return;
     double y;
     int p;
-    split_exp(x[i], tab, y, p);
+    split_exp(x[i], tab, fp64_ops(tab), y, p);
     y_mant[i] = y;
     y_pow[i] = p;
     y_scaled[i] = scale_pow2(v[i], k[i]);
 }
 
 // (flog's domain is x >= 2: see its comment)
-__global__ void selftest_log_kernel(long long n, const double *x, const double2 *tab, double *y_log,
-                                    double *y_log_ref) {
+__global__ void selftest_log_kernel(long long n, const double *x, const double2 *tab, const double *exp_tab,
+                                    double *y_log, double *y_log_ref) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    y_log[i] = flog(x[i], tab);
+    y_log[i] = flog(x[i], tab, exp_tab, fp64_ops(exp_tab));
     y_log_ref[i] = log(x[i]);
 }
 
@@ -49,36 +50,42 @@ __global__ void selftest_log_kernel(long long n, const double *x, const double2 
 
 using namespace chem;
 
+static int upload_exp_table(double **d_tab) {
+    std::vector<double> tab;
+    fill_exp_table(tab);
+    cudaError_t ce = cudaMalloc(d_tab, sizeof(double) * tab.size());
+    if (ce != cudaSuccess) return fail(CHEM_E_OOM, "self-test table");
+    ce = cudaMemcpy(*d_tab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice);
+    if (ce != cudaSuccess) {
+        cudaFree(*d_tab);
+        return cuda_fail(ce, "self-test table");
+    }
+    return CHEM_OK;
+}
+
 extern "C" int chem_selftest_log(int64_t n, const double *x, double *y_log, double *y_log_ref, void *stream) {
     if (n < 0 || !x || !y_log || !y_log_ref) return fail(CHEM_E_INVALID_ARG, "NULL argument");
     if (n == 0) return CHEM_OK;
     std::vector<double> tab;
     fill_log_table(tab);
-    double *d_tab = nullptr;
+    double *d_tab = nullptr, *d_exp = nullptr;
+    const int rc = upload_exp_table(&d_exp);
+    if (rc) return rc;
     cudaError_t ce = cudaMalloc(&d_tab, sizeof(double) * tab.size());
-    if (ce != cudaSuccess) return fail(CHEM_E_OOM, "self-test table");
+    if (ce != cudaSuccess) {
+        cudaFree(d_exp);
+        return fail(CHEM_E_OOM, "self-test table");
+    }
     ce = cudaMemcpy(d_tab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice);
     if (ce == cudaSuccess) {
         selftest_log_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
-            n, x, reinterpret_cast<const double2 *>(d_tab), y_log, y_log_ref);
+            n, x, reinterpret_cast<const double2 *>(d_tab), d_exp, y_log, y_log_ref);
         ce = cudaGetLastError();
         if (ce == cudaSuccess) ce = cudaStreamSynchronize((cudaStream_t)stream);
     }
     cudaFree(d_tab);
+    cudaFree(d_exp);
     if (ce != cudaSuccess) return cuda_fail(ce, "self-test");
-    return CHEM_OK;
-}
-
-static int upload_exp_table(double **d_tab) {
-    std::vector<double> tab(kExpTab);
-    for (int j = 0; j < kExpTab; ++j) tab[j] = (double)std::exp2l((long double)j / kExpTab);
-    cudaError_t ce = cudaMalloc(d_tab, sizeof(double) * kExpTab);
-    if (ce != cudaSuccess) return fail(CHEM_E_OOM, "self-test table");
-    ce = cudaMemcpy(*d_tab, tab.data(), sizeof(double) * kExpTab, cudaMemcpyHostToDevice);
-    if (ce != cudaSuccess) {
-        cudaFree(*d_tab);
-        return cuda_fail(ce, "self-test table");
-    }
     return CHEM_OK;
 }
 
@@ -103,13 +110,11 @@ extern "C" int chem_selftest_math(int64_t n, const double *x, double *y_exp, dou
     if (n < 0 || !x || !y_exp || !y_exp_ref || !y_rcp || !y_rcp_ref)
         return fail(CHEM_E_INVALID_ARG, "NULL argument");
     if (n == 0) return CHEM_OK;
-    std::vector<double> tab(kExpTab);
-    for (int j = 0; j < kExpTab; ++j) tab[j] = (double)std::exp2l((long double)j / kExpTab);
     double *d_tab = nullptr;
-    cudaError_t ce = cudaMalloc(&d_tab, sizeof(double) * kExpTab);
-    if (ce != cudaSuccess) return fail(CHEM_E_OOM, "self-test table");
-    ce = cudaMemcpy(d_tab, tab.data(), sizeof(double) * kExpTab, cudaMemcpyHostToDevice);
-    if (ce == cudaSuccess) {
+    const int rc = upload_exp_table(&d_tab);
+    if (rc) return rc;
+    cudaError_t ce = cudaSuccess;
+    {
         selftest_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(n, x, d_tab, y_exp, y_exp_ref,
                                                                                       y_rcp, y_rcp_ref);
         ce = cudaGetLastError();
