@@ -366,12 +366,12 @@ int chem_server_stats(chem_server_t s, chem_server_stats_t *out);
  * first column with a zero or non-finite pivot (elimination continues past
  * it; that system's A and x are then meaningless).  Arithmetic, layout and
  * kernel by method:
- *   CHEM_LU_GLOBAL      A[(i*n + j)*n_sys + k], b[i*n_sys + k] (interleaved);
- *                       the matrices stay in HBM (the paper's global-memory
- *                       approach): a thread per system when the systems
- *                       fill the GPU, else a block of warps per 32 systems
- *                       sharing each step's rows.  Every step explicitly
- *                       rounded in the scalar order (multiplier a_ij / a_jj,
+ *   CHEM_LU_GLOBAL      A[(i*n + j)*n_sys + k], b[i*n_sys + k] (interleaved).
+ *                       Medium systems are staged in shared memory; small
+ *                       ones and those beyond it (n > 169) stay in HBM (the
+ *                       paper's global-memory approach).  Every step
+ *                       explicitly rounded in the scalar order (multiplier
+ *                       a_ij / a_jj,
  *                       update a_ik - l a_jk without contraction): factors,
  *                       pivots and x equal a scalar elimination with
  *                       row-by-row substitutions bit for bit.
@@ -379,12 +379,12 @@ int chem_server_stats(chem_server_t s, chem_server_stats_t *out);
  *                       multipliers a_ij times one reciprocal of the pivot,
  *                       updates and substitutions as fused multiply-adds;
  *                       equal to the scalar elimination to rounding.
- *   CHEM_LU_ONCHIP      A[(k*n + i)*n + j], b[k*n + i] (contiguous); one warp
- *                       per system, the matrix in shared memory
+ *   CHEM_LU_ONCHIP      A[(k*n + i)*n + j], b[k*n + i] (contiguous); 8 to 256
+ *                       threads per system, the matrix in shared memory
  *                       (CHEM_E_UNSUPPORTED when n*(n+1) doubles do not
  *                       fit); factors and pivots bit for bit as
  *                       CHEM_LU_GLOBAL, x to rounding (the back
- *                       substitution runs by columns across the warp).
+ *                       substitution runs by columns across the threads).
  * Device pointers; asynchronous on `stream`; CHEM_E_INVALID_ARG for an
  * unknown method, n out of range, n_sys < 0 or a null A or b. */
 #define CHEM_LU_GLOBAL     0
