@@ -769,63 +769,7 @@ unsigned long long *next_counter(Handle *h) {
 
 using namespace chem;
 
-// ---------------------------------------------------------------------------
-// small kernels: state from (T, P, Y) and temperature of given states
 namespace chem {
-
-__global__ void state_from_tpy_kernel(DeviceMech m, long long n, long long ld, const double *T,
-                                      const double *P, const double *Y, double *rho, double *e) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double Ti = T[i], invT = 1.0 / Ti;
-    double invW = 0.0;
-    for (int s = 0; s < m.ns; ++s) invW += Y[(size_t)s * ld + i] * m.sp[s * kSpStride + 1];
-    const double rt = P[i] / (kR * Ti * invW);
-    double ei = 0.0;
-    for (int s = 0; s < m.ns; ++s) {
-        const double rs = rt * Y[(size_t)s * ld + i];
-        rho[(size_t)s * ld + i] = rs;
-        const auto th = coef_row(m.thermo, m.ns, s, Ti > m.tmid[s] ? 1 : 0);
-        const double hRT = th[0] + Ti * (th[5] + Ti * (th[6] + Ti * (th[7] + Ti * th[8]))) + th[9] * invT;
-        ei += rs * (m.sp[s * kSpStride + 2] * Ti * (hRT - 1.0) - m.sp[s * kSpStride + 3]);
-    }
-    e[i] = ei;
-}
-
-__global__ void temperature_kernel(DeviceMech m, long long n, long long ld, const double *rho,
-                                   const double *e, const double *Tg, double *Tout) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double lo = kTlo, hi = kThi, T = Tg ? Tg[i] : 1500.0;
-    if (!(T > lo && T < hi)) T = 1500.0;
-    const double ei = e[i];
-    bool ok = false;
-    for (int it = 1; it <= kTmaxIter; ++it) {
-        const double invT = 1.0 / T;
-        double f = 0.0, fp = 0.0;
-        for (int s = 0; s < m.ns; ++s) {
-            const auto th = coef_row(m.thermo, m.ns, s, T > m.tmid[s] ? 1 : 0);
-            const double cpR = th[0] + T * (th[1] + T * (th[2] + T * (th[3] + T * th[4])));
-            const double hRT = th[0] + T * (th[5] + T * (th[6] + T * (th[7] + T * th[8]))) + th[9] * invT;
-            const double RM = m.sp[s * kSpStride + 2];
-            const double r = rho[(size_t)s * ld + i];
-            f += r * (RM * T * (hRT - 1.0) - m.sp[s * kSpStride + 3]);
-            fp += r * RM * (cpR - 1.0);
-        }
-        f -= ei;
-        if (f == 0.0) { ok = true; break; }
-        if (f > 0.0) hi = T; else lo = T;
-        double Tn = T - f / fp;
-        if (!(Tn > lo && Tn < hi)) Tn = 0.5 * (lo + hi);
-        const double dT = Tn - T;
-        T = Tn;
-        if (fabs(dT) <= kTtol * T) {
-            ok = !(T <= kTlo * (1.0 + 1e-9) || T >= kThi * (1.0 - 1e-9));
-            break;
-        }
-    }
-    Tout[i] = ok ? T : NAN;
-}
 
 static_assert(kSchedWords == CHEM_SCHEDULE_WORDS, "schedule record size");
 static_assert(kSubstepStates == CHEM_SUBSTEP_STATES, "substep-state record size");
@@ -1112,38 +1056,6 @@ int chem_advance_host(chem_handle_t hh, int64_t n_cells, int64_t ld, double *rho
     if (ce != cudaSuccess) return cuda_fail(ce, "device-to-host copy");
     ce = cudaStreamSynchronize(st);
     if (ce != cudaSuccess) return cuda_fail(ce, "synchronising the step");
-    return CHEM_OK;
-}
-
-int chem_state_from_tpy(chem_handle_t hh, int64_t n, int64_t ld, const double *T, const double *P,
-                        const double *Y, double *rho_s, double *e, void *stream) {
-    Handle *h = hh;
-    if (!h || !T || !P || !Y || !rho_s || !e) return fail(CHEM_E_INVALID_ARG, "NULL argument");
-    if (n < 0 || (ld != 0 && ld < n)) return fail(CHEM_E_INVALID_ARG, "sizes");
-    if (n == 0) return CHEM_OK;
-    if (ld == 0) ld = n;
-    const int bs = 128;
-    state_from_tpy_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, (cudaStream_t)stream>>>(h->mech, n, ld, T, P, Y,
-                                                                                          rho_s, e);
-    cudaError_t ce = cudaGetLastError();
-    if (ce != cudaSuccess) return cuda_fail(ce, "state_from_tpy launch");
-    h->launches.fetch_add(1);
-    return CHEM_OK;
-}
-
-int chem_temperature(chem_handle_t hh, int64_t n, int64_t ld, const double *rho_s, const double *e,
-                     const double *T_guess, double *T_out, void *stream) {
-    Handle *h = hh;
-    if (!h || !rho_s || !e || !T_out) return fail(CHEM_E_INVALID_ARG, "NULL argument");
-    if (n < 0 || (ld != 0 && ld < n)) return fail(CHEM_E_INVALID_ARG, "sizes");
-    if (n == 0) return CHEM_OK;
-    if (ld == 0) ld = n;
-    const int bs = 128;
-    temperature_kernel<<<(unsigned)((n + bs - 1) / bs), bs, 0, (cudaStream_t)stream>>>(h->mech, n, ld, rho_s, e,
-                                                                                      T_guess, T_out);
-    cudaError_t ce = cudaGetLastError();
-    if (ce != cudaSuccess) return cuda_fail(ce, "temperature launch");
-    h->launches.fetch_add(1);
     return CHEM_OK;
 }
 

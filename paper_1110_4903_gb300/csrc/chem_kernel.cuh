@@ -42,6 +42,7 @@
 
 #include <type_traits>
 
+#include "chem_fp64.cuh"
 #include "chem_internal.h"
 
 namespace chem {
@@ -65,32 +66,6 @@ enum SlotAction : int {
     kFailSubstep = 2,
     kEmitCell = 3
 };
-
-// The FP64 pipe takes a warp's fused multiply-add with three register
-// operands every 16 cycles, but an addition, a multiplication or anything
-// with a constant operand only every 19 (measured, 4 to 20 warps on an SM).
-// So sums and products are written as fused multiply-adds with a 1 and a -0
-// in registers (the same results, signed zeros included), and constants come
-// from a table in global memory.  The loads are volatile: the compiler must
-// not see the values, nor keep all of them in registers.
-struct Fp64Ops {
-    double one, nz;   // 1 and -0
-    __device__ __forceinline__ double add(double a, double b) const { return __fma_rn(a, one, b); }
-    __device__ __forceinline__ double sub(double a, double b) const { return __fma_rn(-b, one, a); }
-    __device__ __forceinline__ double mul(double a, double b) const { return __fma_rn(a, b, nz); }
-};
-__device__ __forceinline__ double2 ld_const2(const double *p) {
-    double2 v;
-    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];"
-                 : "=d"(v.x), "=d"(v.y)
-                 : "l"(__cvta_generic_to_global(p)));
-    return v;
-}
-// (tab: the exp table, which the constants follow)
-__device__ __forceinline__ Fp64Ops fp64_ops(const double *tab) {
-    const double2 v = ld_const2(tab + kConstOne);
-    return Fp64Ops{v.x, v.y};
-}
 
 template <int G>
 struct Grp {
@@ -149,52 +124,11 @@ struct Grp {
     }
 };
 
-// Conversions between FP64 and FP32 on the integer pipe: on this part a
-// conversion instruction occupies the FP64 pipe as long as a DFMA does.
-// FP64 -> FP32 rounds toward zero; magnitudes below the smallest normal
-// float give a signed zero, above the largest an infinity; NaN stays NaN.
-__device__ __forceinline__ float d2f_rz(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
-    const unsigned sign = hi & 0x80000000u;
-    const int e = (int)((hi >> 20) & 0x7ffu) - 896;
-    const unsigned man = ((hi & 0xfffffu) << 3) | (lo >> 29);
-    unsigned f = sign | ((unsigned)e << 23) | man;
-    if (e <= 0) f = sign;
-    if (e >= 255) f = sign | 0x7f800000u | ((e == 1151 && ((hi & 0xfffffu) | lo)) ? 0x400000u : 0u);
-    return __uint_as_float(f);
-}
-// FP32 -> FP64, exact for normal floats and infinities (NaN stays NaN,
-// subnormal floats give a signed zero).
-__device__ __forceinline__ double f2d_alu(float v) {
-    const unsigned u = __float_as_uint(v);
-    const unsigned sign = u & 0x80000000u, e = (u >> 23) & 0xffu, man = u & 0x7fffffu;
-    unsigned hi = sign | ((e + 896u) << 20) | (man >> 3);
-    unsigned lo = man << 29;
-    if (e == 0) {
-        hi = sign;
-        lo = 0u;
-    }
-    if (e == 255u) hi = sign | 0x7ff00000u | (man >> 3);
-    return __hiloint2double((int)hi, (int)lo);
-}
 template <typename JT> __device__ __forceinline__ JT to_jt(double v);
 template <> __device__ __forceinline__ double to_jt<double>(double v) { return v; }
 template <> __device__ __forceinline__ float to_jt<float>(double v) { return d2f_rz(v); }
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return f2d_alu(v); }
-
-// Order of doubles by their bit patterns (integer pipe): exact for a >= 0
-// against b > 0; a negative a counts as smaller, a NaN a as larger.
-__device__ __forceinline__ bool bits_gt(double a, double b) {
-    return __double_as_longlong(a) > __double_as_longlong(b);
-}
-__device__ __forceinline__ bool bits_lt(double a, double b) {
-    return __double_as_longlong(a) < __double_as_longlong(b);
-}
-__device__ __forceinline__ bool finite_bits(double v) {
-    return ((unsigned)((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffu) != 0x7ffu;
-}
 
 // Argmax over a whole warp (one cell per warp) with redux.sync: the largest
 // key, the lowest index on ties, as the shuffle tree gives it.  FP64 keys
@@ -228,24 +162,6 @@ __device__ __forceinline__ bool key_is_inf(unsigned k) { return k >= 0x7f800000u
 template <typename JT>
 using PivotKey = decltype(abs_key(JT(0)));
 
-// Reciprocal: the hardware approximation r refined with its residual
-// e = 1 - a r as r (1 + e + e^2), whose error is e^3 (the approximation is
-// good to about 2^-23, so below FP64 rounding): three FP64 operations.
-__device__ __forceinline__ double frcp(double a, const Fp64Ops &op) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    const double e = fma(-a, r, op.one);
-    return fma(r, fma(e, e, e), r);
-}
-// One Newton step only (relative error about 1e-14): for reciprocals that
-// scale a convergence ratio or the temperature recovery's Newton step, never
-// a rate, an energy or the elimination.
-__device__ __forceinline__ double frcp1(double a, const Fp64Ops &op) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    const double e = fma(-a, r, op.one);
-    return fma(r, e, r);
-}
 // FP32 reciprocal of the pivot: the hardware approximation (within an ulp or
 // two), enough for an elimination whose result Newton refines in FP64.
 __device__ __forceinline__ float frcp(float a) {
@@ -382,11 +298,6 @@ __device__ __forceinline__ double flog(double x, const double2 *tab, const doubl
 __device__ __forceinline__ double nasa_s(const CoefRow<double> &th, double T, double lnT, const Fp64Ops &op) {
     return op.add(fma(th[0], lnT, op.mul(T, fma(T, fma(T, fma(T, th[12], th[11]), th[10]), th[1]))), th[13]);
 }
-// range of species s at T (1: T > T_mid, the high range)
-__device__ __forceinline__ int thermo_range(const DeviceMech &m, int s, long long Tbits) {
-    return Tbits > __ldg(reinterpret_cast<const long long *>(m.tmid) + s) ? 1 : 0;
-}
-
 // Temperature recovery from (rho_s, e) for every slot whose `need` is set:
 // Newton on sum_s rho_s e_s^sens(T) = e, safeguarded by bisection on
 // [kTlo, kThi], stop at |dT| <= kTtol T (Eq. 3 with the kinetic energy left to
