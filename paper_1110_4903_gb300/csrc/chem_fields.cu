@@ -146,11 +146,16 @@ __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m
             hi = T;
         else
             lo = T;
-        double Tn = T - f / fp;
-        if (!(Tn > lo && Tn < hi)) Tn = 0.5 * (lo + hi);
-        const double dT = Tn - T;
+        // (a step within the tolerance ends the iteration wherever it lands:
+        // below half an ulp it leaves T at an end of the bracket)
+        double Tn = T - f / fp, dT = Tn - T;
+        const double tol = kTtol * T;
+        if (!(fabs(dT) <= tol) && !(Tn > lo && Tn < hi)) {
+            Tn = 0.5 * (lo + hi);
+            dT = Tn - T;
+        }
         T = Tn;
-        if (fabs(dT) <= kTtol * T) {
+        if (fabs(dT) <= tol) {
             ok = !(T <= kTlo * (1.0 + 1e-9) || T >= kThi * (1.0 - 1e-9));
             break;
         }

@@ -356,12 +356,18 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
                     hi = T;
                 else
                     lo = T;
-                double Tn = fma(-f, rfp, T);
-                if (!(bits_gt(Tn, lo) && bits_lt(Tn, hi))) Tn = 0.5 * (lo + hi);
-                const double dT = op.sub(Tn, T);
-                T = Tn;
+                // A step within the tolerance ends the recovery wherever it
+                // lands: below half an ulp it leaves T at an end of the
+                // bracket, and bisecting from there would start all over
+                double Tn = fma(-f, rfp, T), dT = op.sub(Tn, T);
+                const double tol = kTtol * T;
                 // (comparisons of non-negative doubles on their bit patterns)
-                if (!bits_gt(fabs(dT), kTtol * T)) {
+                if (bits_gt(fabs(dT), tol) && !(bits_gt(Tn, lo) && bits_lt(Tn, hi))) {
+                    Tn = 0.5 * (lo + hi);
+                    dT = op.sub(Tn, T);
+                }
+                T = Tn;
+                if (!bits_gt(fabs(dT), tol)) {
                     done = true;
                     ok = bits_gt(T, kTlo * (1.0 + 1e-9)) && bits_lt(T, kThi * (1.0 - 1e-9));
                 }
