@@ -253,6 +253,7 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
             for (int i = 1; i <= 4; ++i) c[6 + i] = (double)(RM * a[i]);
             float *cf = &t.tpoly_f[((size_t)s * 2 + rg) * kTpolyFStride];
             for (int i = 0; i <= 4; ++i) cf[i] = (float)c[6 + i];
+            for (int i = 0; i <= 5; ++i) cf[5 + i] = (float)c[i];
         }
     // dense stoichiometry
     std::vector<int> nuR((size_t)nr * ns, 0), nuP((size_t)nr * ns, 0);

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kFieldThreads) state_from_tpy_kernel(DeviceMec
 }
 
 // Temperature of (rho, e): Newton on sum_s rho_s e_s^sens(T) = e safeguarded by
-// bisection on [kTlo, kThi], stop at |dT| <= kTtol T, as in the step.  Without
+// bisection on [kTlo, kThi], ended as in the step.  Without
 // a guess, and where no density is negative (so that e(T) is increasing and
 // has one root), Newton runs in FP32 first, at a sixty-fourth of the cost: from
 // 1500 K the FP64 iterations were six or seven, from there they are three.
@@ -146,11 +146,11 @@ __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m
             hi = T;
         else
             lo = T;
-        // (a step within the tolerance ends the iteration wherever it lands:
-        // below half an ulp it leaves T at an end of the bracket)
         double Tn = T - f / fp, dT = Tn - T;
-        const double tol = kTtol * T;
-        if (!(fabs(dT) <= tol) && !(Tn > lo && Tn < hi)) {
+        const bool inside = Tn > lo && Tn < hi;
+        const double tol = (inside ? kTstep : kTtol) * T;
+        // (a step below half an ulp leaves T at an end of the bracket)
+        if (!inside && !(fabs(dT) <= tol)) {
             Tn = 0.5 * (lo + hi);
             dT = Tn - T;
         }

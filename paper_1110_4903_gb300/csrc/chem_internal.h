@@ -20,7 +20,8 @@ constexpr double kLnPaOverR = 9.408091968961747;   // ln(kPa / kR), rounded from
 constexpr double kTlo = 200.0;         // temperature-recovery bracket, K
 constexpr double kThi = 6000.0;
 constexpr int kTmaxIter = 50;          // temperature-recovery iterations
-constexpr double kTtol = 1e-13;        // |dT| <= kTtol * T ends the recovery
+constexpr double kTtol = 1e-13;        // |dT| <= kTtol * T ends the recovery,
+constexpr double kTstep = 1e-9;        //   a Newton step inside the bracket at kTstep * T
 
 // Polynomial tables are stored coefficient-major, so that the lanes of a
 // warp, which hold consecutive species, read consecutive words: coefficient
@@ -41,9 +42,9 @@ constexpr int kThermoStride = 16;
 //   0..5  e_s(T) - e_f,s = c0 + c1 T + ... + c5 T^5  (c0 = R/M a6 - e_f,
 //         c1 = R/M (a1 - 1), c_i = R/M a_i / i for i = 2..5)
 //   6..10 c_v,s(T) = R/M (cp/R - 1) = d0 + d1 T + ... + d4 T^4
-// and an FP32 copy of d0..d4 (8 coefficients).
+// and an FP32 copy of d0..d4, c0..c5 (12 coefficients).
 constexpr int kTpolyStride = 12;
-constexpr int kTpolyFStride = 8;
+constexpr int kTpolyFStride = 12;
 
 // Species table row (4 doubles): M, 1/M, R/M, e_f = e_s(T_ref).
 constexpr int kSpStride = 4;
@@ -131,7 +132,7 @@ struct DeviceMech {
     const double *thermo;       // [16][2][ns] (coefficient-major, above)
     const double *tmid;         // [ns] (positive: compared as integers)
     const double *tpoly;        // [12][2][ns] energy and heat-capacity polynomials
-    const float *tpoly_f;       // [8][2][ns] heat-capacity polynomial in FP32
+    const float *tpoly_f;       // [12][2][ns] heat-capacity and energy polynomials in FP32
     const double *sp;           // [ns][4]
     const double *rxn_d;        // [nr][4] ln A (SI), beta, E/R, sum nu
     const int *rxn_f;           // [nr][2]

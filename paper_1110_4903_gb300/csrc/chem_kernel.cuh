@@ -300,14 +300,19 @@ __device__ __forceinline__ double nasa_s(const CoefRow<double> &th, double T, do
 }
 // Temperature recovery from (rho_s, e) for every slot whose `need` is set:
 // Newton on sum_s rho_s e_s^sens(T) = e, safeguarded by bisection on
-// [kTlo, kThi], stop at |dT| <= kTtol T (Eq. 3 with the kinetic energy left to
-// the flux stage).  Uniform across the warp.
+// [kTlo, kThi] (Eq. 3 with the kinetic energy left to the flux stage).  A
+// Newton step of at most kTstep T ends it: with the derivative good to 1e-7
+// the temperature is then good to 1e-16, and another pass would only confirm
+// that.  Uniform across the warp.
+//   `cold` slots have no guess: where no density is negative (so that e(T) is
+// increasing and has one root) three Newton steps in FP32 find one, from
+// which two FP64 passes suffice instead of six.
 //   The energies come from the multiplied-out polynomials (five DFMA per
 //   species, no 1/T); with F32 the derivative sum c_v is formed in FP32, which
 //   changes the Newton steps by a relative 1e-7 and not the root.
 template <int G, bool F32>
 __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab, const double *x, int sl, bool need,
-                                          double guess, double &T_out, bool &ok) {
+                                          bool cold, double guess, double &T_out, bool &ok) {
     const int ns = m.ns;
     const Fp64Ops op = fp64_ops(tab);
     double lo = kTlo, hi = kThi, T = guess;
@@ -315,6 +320,30 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
     bool done = !need;
     ok = false;
     const double e = x[ns];
+    if (__any_sync(kFull, cold)) {
+        float Tf = 1500.f;
+        int neg = 0;
+#pragma unroll 1
+        for (int it = 0; it < 3; ++it) {
+            const long long Tb = __double_as_longlong(f2d_alu(Tf));
+            float f = 0.f, fp = 0.f;
+#pragma unroll 1
+            for (int s = sl; s < ns; s += G) {
+                const auto d = coef_row(m.tpoly_f, ns, s, thermo_range(m, s, Tb));
+                const float r = d2f_rz(x[s]);
+                neg |= r < 0.f;
+                f = fmaf(r, fmaf(fmaf(fmaf(fmaf(fmaf(d[10], Tf, d[9]), Tf, d[8]), Tf, d[7]), Tf, d[6]), Tf, d[5]), f);
+                fp = fmaf(r, fmaf(fmaf(fmaf(fmaf(d[4], Tf, d[3]), Tf, d[2]), Tf, d[1]), Tf, d[0]), fp);
+            }
+            f = Grp<G>::sum(f) - d2f_rz(e);
+            fp = Grp<G>::sum(fp);
+            Tf -= __fdividef(f, fp);
+            Tf = fminf(fmaxf(Tf, (float)kTlo), (float)kThi);   // (a NaN goes to the lower end)
+        }
+        neg = Grp<G>::any(neg);
+        const double Ts = f2d_alu(Tf);
+        if (cold && !neg && bits_gt(Ts, lo) && bits_lt(Ts, hi)) T = Ts;
+    }
 #pragma unroll 1
     for (int it = 1; it <= kTmaxIter; ++it) {
         if (!__any_sync(kFull, !done)) break;
@@ -356,13 +385,13 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
                     hi = T;
                 else
                     lo = T;
-                // A step within the tolerance ends the recovery wherever it
-                // lands: below half an ulp it leaves T at an end of the
-                // bracket, and bisecting from there would start all over
-                double Tn = fma(-f, rfp, T), dT = op.sub(Tn, T);
-                const double tol = kTtol * T;
                 // (comparisons of non-negative doubles on their bit patterns)
-                if (bits_gt(fabs(dT), tol) && !(bits_gt(Tn, lo) && bits_lt(Tn, hi))) {
+                double Tn = fma(-f, rfp, T), dT = op.sub(Tn, T);
+                const bool inside = bits_gt(Tn, lo) && bits_lt(Tn, hi);
+                const double tol = (inside ? kTstep : kTtol) * T;
+                // (a step below half an ulp leaves T at an end of the bracket:
+                // it ends the recovery, bisecting would start it all over)
+                if (!inside && bits_gt(fabs(dT), tol)) {
                     Tn = 0.5 * (lo + hi);
                     dT = op.sub(Tn, T);
                 }
@@ -1685,7 +1714,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
             if (!__any_sync(kFull, needT || act != kNoAction)) break;
             double Tr = T;
             bool ok = false;
-            recover_T<G, sizeof(JT) == 4>(m, tab, sm.x, sl, needT, T, Tr, ok);
+            recover_T<G, sizeof(JT) == 4>(m, tab, sm.x, sl, needT, state == kInitT && (Q || !b.T_in), T, Tr, ok);
             int neg = 0;
 #pragma unroll 1
             for (int i = sl; i < ns; i += G)
