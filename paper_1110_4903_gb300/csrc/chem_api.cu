@@ -180,7 +180,7 @@ struct HostTables {
         std::vector<int> j_d;
         std::vector<double> j_c;
     } lay[kLayouts];
-    int nD = 0, nD_F1 = 0, nD_B1 = 0, nJ = 0, nJ_nz = 0, n_items = 0, ntb = 0;
+    int nD = 0, nD_F1 = 0, nD_1 = 0, nD_F2 = 0, nD_2 = 0, nJ = 0, nJ_nz = 0, n_items = 0, ntb = 0;
 };
 
 // {1/F, ln F} at F = 1 + j/kLogTab, j = 0..kLogTab, rounded from extended
@@ -346,10 +346,10 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
         t.d_cef.push_back((float)e.alpha1);
         t.d_i1.push_back(e.fa | (e.fb << 8) | (e.ba << 16) | (e.bb << 24));
     }
-    // the FP64 kernel's order: entries that take one multiplication first
+    // the FP64 kernel's order (chem_internal.h)
     auto kind64 = [&](const DEnt &e) {
-        const bool one = e.vf + e.vb == 1 && (e.vf ? e.fb : e.bb) == SENT;
-        return one ? (e.vf ? 0 : 1) : 2 + 4 * e.grp + std::max(e.vf, e.vb);
+        if (e.vf + e.vb != 1) return 4 + 4 * e.grp + std::max(e.vf, e.vb);
+        return ((e.vf ? e.fb : e.bb) == SENT ? 0 : 2) + (e.vf ? 0 : 1);
     };
     std::vector<int> ord64(t.nD), pos64(t.nD);
     for (int j = 0; j < t.nD; ++j) ord64[j] = j;
@@ -358,7 +358,9 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
         const DEnt &e = ents[ord64[j]];
         pos64[ord64[j]] = j;
         if (kind64(e) <= 0) t.nD_F1++;
-        if (kind64(e) <= 1) t.nD_B1++;
+        if (kind64(e) <= 1) t.nD_1++;
+        if (kind64(e) <= 2) t.nD_F2++;
+        if (kind64(e) <= 3) t.nD_2++;
         t.d_pk64.push_back(make_int2(t.d_i0[ord64[j]], t.d_i1[ord64[j]]));
         t.d_ce.push_back(e.alpha1);
     }
@@ -660,7 +662,9 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
     m.ntb = t.ntb;
     m.nD = t.nD;
     m.nD_F1 = t.nD_F1;
-    m.nD_B1 = t.nD_B1;
+    m.nD_1 = t.nD_1;
+    m.nD_F2 = t.nD_F2;
+    m.nD_2 = t.nD_2;
     m.nJ = t.nJ;
     m.nJ_nz = t.nJ_nz;
     m.n_items = t.n_items;

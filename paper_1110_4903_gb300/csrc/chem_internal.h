@@ -80,9 +80,9 @@ constexpr int kLogTab = 128;
 // progress rate Q_r depends on, holding dQ_r/drho_k without the all-ones
 // third-body part.  They are sorted into four groups: reactant-only,
 // product-only, both sides, efficiency-only.  The FP64 kernel keeps them in an
-// order of its own (d_pk64): [0, F1) reactant-only of order 1 with at most one
-// remaining factor, [F1, B1) the same for products, then the others, by
-// group and order.
+// order of its own (d_pk64): those of order 1 on one side with at most one
+// remaining factor, reactants [0, F1) and products [F1, 1), with two, [1, F2)
+// and [F2, 2), then the others by group and order.
 //   d_pk = {r | nu'_rk << 16 | nu''_rk << 20,
 //           fa | fb << 8 | ba << 16 | bb << 24  (the remaining factors of
 //                d(prod c)/dc_k on each side, sentinel ns if none)}
@@ -125,7 +125,8 @@ __host__ __device__ constexpr int layout_index(int G) {
 struct DeviceMech {
     int ns, nr;
     int ntb;                    // third-body reactions: the first ntb (internal order)
-    int nD, nD_F1, nD_B1;       // D entries; ends of the FP64 order's first groups
+    int nD;                     // D entries; ends of the FP64 order's first groups:
+    int nD_F1, nD_1, nD_F2, nD_2;
     int nJ;                     // Jacobian entries gathered: ns*ns (species rows and columns)
     int nJ_nz;                  //   of which the first nJ_nz have reaction terms (longest list first)
     int n_items;                // species-gather work items

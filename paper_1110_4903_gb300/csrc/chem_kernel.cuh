@@ -760,11 +760,12 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             sm.cJ[s] = to_jt<JT>(ci);
             sm.hJ[s] = hJs;
         } else {
-            const double es = fma(op.mul(RM, T), op.sub(hRT, op.one), -__ldg(spr + 3));
+            const double hm1 = op.sub(hRT, op.one);
+            const double es = fma(op.mul(RM, T), hm1, -__ldg(spr + 3));
             const auto c = coef_row(m.tpoly, ns, s, rg);
             const double cv = fma(fma(fma(fma(c[10], T, c[9]), T, c[8]), T, c[7]), T, c[6]);
             rhocv = fma(xs, cv, rhocv);
-            sm.hRT[s] = hRT;
+            sm.hRT[s] = hm1;
             sm.es[s] = es;
         }
     }
@@ -862,7 +863,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         }
         const double rev = op.mul(kb, Pb), fwd = f32 ? 0.0 : op.mul(kf, Pf);
         const double q = f32 ? fma(kf, Pf, -rev) : op.sub(fwd, rev);
-        sm.Q[r] = op.mul(CM, q);   // in the D region until phase 4
+        sm.Q[r] = f32 || tb ? op.mul(CM, q) : q;   // in the D region until phase 4
         if (f32) {
             // Jacobian-only quantities in FP32 from FP32 copies
             const float *rf = m.rxn_df + (size_t)r * kRxnDStride;
@@ -886,15 +887,19 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             }
             sm.dQdT[r] = A1v * PfJ * dlnkf - A2v * PbJ * (dlnkf - dlnKc);
         } else {
+            // Jacobian-only quantities, scaled by -h here where it costs
+            // nothing: -h C_M k_f, -h C_M k_b, -h q_tb, and -h T dQ/dT (the
+            // species' sums take the 1/T)
+            //   T dln k_f/dT = beta + E/RT,
+            //   T dln k_b/dT = that less sum nu (h/RT - 1)
             const double hb = op.add(sm.hRT[b0], sm.hRT[b1]), ha = op.add(sm.hRT[a0], sm.hRT[a1]);
             const double sh = s3 ? op.sub(op.add(hb, sm.hRT[b2]), op.add(ha, sm.hRT[a2])) : op.sub(hb, ha);
-            if (r < m.ntb) sm.qtb[r] = (JT)q;
-            sm.A1[r] = (JT)op.mul(CM, kf);
-            sm.A2[r] = (JT)op.mul(CM, kb);
-            const double dlnkf = fma(EaRT, invT, op.mul(beta, invT));
-            // (d ln K_b/dT = d ln K_f/dT - (sh - dnu) / T)
-            const double dlnkb = fma(-op.sub(sh, dnu), invT, dlnkf);
-            sm.dQdT[r] = (JT)op.mul(CM, fma(fwd, dlnkf, -op.mul(rev, dlnkb)));
+            const double CMh = tb ? op.mul(CM, -h) : -h;
+            if (r < m.ntb) sm.qtb[r] = (JT)op.mul(q, -h);
+            sm.A1[r] = (JT)op.mul(CMh, kf);
+            sm.A2[r] = (JT)op.mul(CMh, kb);
+            const double dlf = op.add(beta, EaRT);
+            sm.dQdT[r] = (JT)op.mul(CMh, fma(fwd, dlf, -op.mul(rev, op.sub(dlf, sh))));
         }
     }
     __syncwarp();
@@ -983,7 +988,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         // right-hand side -F_s = -(x_s - x0_s - h wdot_s), FP64 until stored
         const double dx = op.sub(sm.x[s], sm.x0[s]);
         sm.rhs[s] = to_jt<JT>(-fma(-h, wds, dx));
-        const JT ws = jmul(MJ, sdq), us = jmul(MJ, squ);
+        // (FP64: -h w and -h u, from sums over -h T dQ/dT and -h q_tb)
+        const JT ws = jmul(f32 ? MJ : (JT)op.mul(M, invT), sdq), us = jmul(MJ, squ);
         sm.w[s] = ws;
         sm.u[s] = us;
         dEt = fma(ef, dx, dEt);
@@ -1005,40 +1011,67 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         const JT *__restrict__ cJv = sm.cJ;
         const JT *__restrict__ qv = sm.qtb;
         JT *__restrict__ Dw = sm.D;
-        auto dval = [&](int j) -> JT {
-            const int2 pk = __ldg(m.d_pk + j);
+        // (descriptors and efficiencies are loaded one trip ahead)
+        struct DEntry {
+            int2 pk;
+            float ce;
+        };
+        auto entry_at = [&](int j) -> DEntry {
+            DEntry d{make_int2(0, 0), 0.f};
+            if (j < m.nD) {
+                d.pk = __ldg(m.d_pk + j);
+                d.ce = __ldg(m.d_cef + j);
+            }
+            return d;
+        };
+        auto dval = [&](const DEntry &en) -> JT {
+            const int2 pk = en.pk;
             const int r = pk.x & 0xffff, vf = (pk.x >> 16) & 15, vb = (pk.x >> 20) & 15, i1 = pk.y;
             const JT fwd = (JT)small_int_to_float(vf) * A1v[r] * (cJv[i1 & 0xff] * cJv[(i1 >> 8) & 0xff]);
             const JT bwd = (JT)small_int_to_float(vb) * A2v[r] * (cJv[(i1 >> 16) & 0xff] * cJv[(i1 >> 24) & 0xff]);
             JT d = (vf ? fwd : (JT)0) - (vb ? bwd : (JT)0);
-            if (r < m.ntb) d = fma((JT)__ldg(m.d_cef + j), qv[r], d);
+            if (r < m.ntb) d = fma((JT)en.ce, qv[r], d);
             return d;
         };
-        int j = sl;
+        DEntry e0 = entry_at(sl), e1 = entry_at(sl + G);
 #pragma unroll 1
-        for (; j + G < m.nD; j += 2 * G) {
-            const JT d0 = dval(j), d1 = dval(j + G);
-            Dw[j] = d0;
-            Dw[j + G] = d1;
+        for (int j = sl; j < m.nD; j += 2 * G) {
+            const DEntry c0 = e0, c1 = e1;
+            e0 = entry_at(j + 2 * G);
+            e1 = entry_at(j + 3 * G);
+            // (past the end: the descriptor 0 reads reaction 0, and is dropped)
+            const JT v0 = dval(c0), v1 = dval(c1);
+            Dw[j] = v0;
+            if (j + G < m.nD) Dw[j + G] = v1;
         }
-        if (j < m.nD) Dw[j] = dval(j);
-    } else
+    } else {
+    int2 npk = sl < m.nD ? __ldg(m.d_pk64 + sl) : make_int2(0, 0);
+    double nce = sl < m.nD ? __ldg(m.d_ce + sl) : 0.0;
 #pragma unroll 1
     for (int j = sl; j < m.nD; j += G) {
         // the FP64 D entries are M_k dQ_r/drho_k as well: integer orders from
         // the descriptor (exact doubles by integer operations), alpha - 1
         // from an 8-byte table, and the gather applies the 1/M_k
-        // (in an order of their own: first those with order 1 and one
-        // remaining factor, one multiplication instead of three)
-        const int2 pk = __ldg(m.d_pk64 + j);
+        // (in an order of their own: first those of order 1 with one
+        // remaining factor, then with two: one and two multiplications
+        // instead of three)
+        const int2 pk = npk;
+        const double ce = nce;
+        if (j + G < m.nD) {
+            npk = __ldg(m.d_pk64 + j + G);
+            nce = __ldg(m.d_ce + j + G);
+        }
         const int r = pk.x & 0xffff, vf = (pk.x >> 16) & 15, vb = (pk.x >> 20) & 15, i1 = pk.y;
         const int fa = i1 & 0xff, fb = (i1 >> 8) & 0xff, ba = (i1 >> 16) & 0xff, bb = (i1 >> 24) & 0xff;
         // (one side's factors, selected without a branch; the reactant side
         // where a species is on both)
+        // (-h M_k dQ_r/drho_k, from -h C_M k)
         double dd;
-        if (j < m.nD_B1) {
-            const bool f = j < m.nD_F1;
-            dd = op.mul(f ? sm.A1[r] : sm.A2[r], sm.c[f ? fa : ba]);
+        if (j < m.nD_2) {
+            const bool f = j < m.nD_F1 || (j >= m.nD_1 && j < m.nD_F2);
+            double A = f ? sm.A1[r] : sm.A2[r];
+            if (j >= m.nD_1) A = op.mul(A, sm.c[f ? fb : bb]);
+            dd = op.mul(A, sm.c[f ? fa : ba]);
             if (!f) dd = -dd;
         } else {
             const bool f = vf > 0;
@@ -1049,7 +1082,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             if (f && vb > 0)
                 dd = fma(A, cc, -op.mul(op.mul(small_pos_int_to_double(vb), sm.A2[r]), op.mul(sm.c[ba], sm.c[bb])));
         }
-        sm.D[j] = r < m.ntb ? (JT)fma(__ldg(m.d_ce + j), (double)sm.qtb[r], dd) : (JT)dd;
+        sm.D[j] = r < m.ntb ? (JT)fma(ce, (double)sm.qtb[r], dd) : (JT)dd;
+    }
     }
     __syncwarp();
     // the per-reaction arrays are dead from here on; the matrix takes their place
@@ -1065,7 +1099,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     //    arithmetic, with one unknown fewer and no energy row to form
     const JT mh = to_jt<JT>(-h);
     {
-        const JT cRE = f32 ? mh * (JT)dTdef * d2f_rz(RE) : (JT)op.mul(op.mul(-h, dTde), RE);
+        const JT cRE = f32 ? mh * (JT)dTdef * d2f_rz(RE) : (JT)op.mul(dTde, RE);   // (FP64: w carries the -h)
 #pragma unroll 1
         for (int i = sl; i < N; i += G) sm.A[ix(i, N)] = fma(sm.w[i], cRE, sm.rhs[i]);
     }
@@ -1168,8 +1202,9 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         }
         __syncwarp();
     } else {
-        // (loads ahead as in the FP32 pass; an addition whose operand is an
-        // exact zero costs an FP64-pipe slot like any other and is skipped)
+        // (loads ahead as in the FP32 pass; w, u and the D entries carry the
+        // -h, the initial values the identity and u: two FP64 operations per
+        // entry beside its terms)
         struct Terms {
             int d[4];
             double c[4];
@@ -1194,40 +1229,30 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             me = mn;
             mn = meta_at(p + 2 * G);
             tn = terms_at(me.x, me.y >> 16);
-            const JT invMk = (JT)__ldg(m.sp + k * kSpStride + 1);
-            const JT J = jmul(sm.w[s], sm.dTdr[k]);
-            JT ua = sm.u[s];
+            const double invMk = __ldg(m.sp + k * kSpStride + 1);
+            // -h w_s dT/drho_k plus the identity; the sum starts from -h u_s
+            // (one accumulator: a warp's FP64 operations do not overlap)
+            const double J = fma((double)sm.w[s], (double)sm.dTdr[k], s == k ? op.one : op.nz);
+            double ua = sm.u[s];
             if (len > 0) {
-                JT a0 = 0, a1 = 0;
 #pragma unroll 1
                 for (;;) {
-                    const JT v0 = Dv[t.d[0]], v1 = Dv[t.d[1]], v2 = Dv[t.d[2]], v3 = Dv[t.d[3]];
+                    const double v0 = Dv[t.d[0]], v1 = Dv[t.d[1]], v2 = Dv[t.d[2]], v3 = Dv[t.d[3]];
                     const Terms tc = t;
                     const int rc = rem;
                     rem -= 4;
                     e += 4 * G;
                     t = terms_at(e, rem);
-                    if (rc >= 4) {
-                        a0 = fma((JT)tc.c[0], v0, a0);
-                        a1 = fma((JT)tc.c[1], v1, a1);
-                        a0 = fma((JT)tc.c[2], v2, a0);
-                        a1 = fma((JT)tc.c[3], v3, a1);
-                    } else {
-                        a0 = fma((JT)tc.c[0], v0, a0);
-                        if (rc > 1) a0 = fma((JT)tc.c[1], v1, a0);
-                        if (rc > 2) a0 = fma((JT)tc.c[2], v2, a0);
-                    }
+                    ua = fma(tc.c[0], v0, ua);
+                    if (rc > 1) ua = fma(tc.c[1], v1, ua);
+                    if (rc > 2) ua = fma(tc.c[2], v2, ua);
+                    if (rc > 3) ua = fma(tc.c[3], v3, ua);
                     if (rem <= 0) break;
                 }
-                if (len >= 4) a0 = jadd(a0, a1);
-                ua = jadd(ua, a0);
             }
             // (D entries scaled by M_k; the FP64 lists' coefficients are nu_rs M_s)
-            sm.A[ix(s, k)] = jmul(mh, fma(invMk, ua, J));
+            sm.A[ix(s, k)] = (JT)fma(invMk, ua, J);
         }
-        __syncwarp();
-#pragma unroll 1
-        for (int i = sl; i < N; i += G) sm.A[ix(i, i)] = jadd(sm.A[ix(i, i)], (JT)op.one);
         __syncwarp();
     }
 
@@ -1297,15 +1322,31 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             const int q0 = (int)(((unsigned)sl * rc) >> 16), dq = (int)(((unsigned)G * rc) >> 16);
             int i = j + 1 + q0, k = j + 1 + (sl - q0 * cols);
             const int di = dq, dk = G - dq * cols;
-#pragma unroll 1
-            for (; e < tot; e += G) {
-                sm.A[i * ldA + k] -= sm.A[i * ldA + j] * sm.A[j * ldA + k];
+            // (two elements per trip, so that their loads overlap)
+            auto next = [&]() {
                 i += di;
                 k += dk;
                 if (k > N) {
                     k -= cols;
                     ++i;
                 }
+            };
+            const JT *rj = sm.A + j * ldA;
+#pragma unroll 1
+            for (; e + G < tot; e += 2 * G) {
+                JT *p0 = sm.A + i * ldA;
+                const int k0 = k;
+                next();
+                JT *p1 = sm.A + i * ldA;
+                const int k1 = k;
+                next();
+                const JT l0 = p0[j], u0 = rj[k0], v0 = p0[k0], l1 = p1[j], u1 = rj[k1], v1 = p1[k1];
+                p0[k0] = fma(-l0, u0, v0);
+                p1[k1] = fma(-l1, u1, v1);
+            }
+            if (e < tot) {
+                JT *p0 = sm.A + i * ldA;
+                p0[k] = fma(-p0[j], rj[k], p0[k]);
             }
         }
         __syncwarp();
