@@ -575,7 +575,8 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
             std::memcpy(&fb, &f, sizeof fb);
             L.j_meta32.push_back(make_int4(mt.x, mt.y >> 16, k * ldc + s, fb));
         }
-        L.j_w.assign(std::max(nw32, 1), 0u);
+        // (the kernel reads whole chunks of four rows, one ahead)
+        L.j_w.assign(nw32 + 8 * G, 0u);
         for (size_t e = 0; e < pos.size(); ++e) L.j_w[pos[e]] = t.j_w[e];
         const int ni = interleave(t.n_items, t.it_ptr, G, L.it_meta, pos, 16, &t.it_id);
         L.sp_w.assign(std::max(ni, 1), 0u);

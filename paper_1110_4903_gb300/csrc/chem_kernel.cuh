@@ -1149,56 +1149,47 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         auto coef = [](unsigned wv) -> float { return __int_as_float((int)(wv & 0xff800000u)); };
         //     Most lists have fewer than four terms, and the table's words
         //     often come from L2: a list's metadata is loaded two entries
-        //     ahead, its first four words one entry ahead, later words one
-        //     chunk ahead, and a chunk's terms are read together.  Terms in
-        //     a whole chunk alternate between two accumulators, those of a
-        //     partial one follow the first.
+        //     ahead, its words one chunk of four ahead.  A branch costs a warp
+        //     some thirty cycles, so the lanes of a pass run the chunks of its
+        //     longest list (lane 0's) together, a missing term being a zero
+        //     times D entry 0 (the table is padded, all reads are in it).
+        //     Terms in a whole chunk alternate between two accumulators, those
+        //     of a partial one follow the first.
         const int nnz = m.nJ_nz;
         auto meta_at = [&](int p) -> int4 { return p < nnz ? __ldg(gl.j_meta32 + p) : make_int4(0, 0, 0, 0); };
-        auto words_at = [&](int e, int rem) -> uint4 {
+        auto words_at = [&](int e) -> uint4 {
             const unsigned *wp = gl.j_w + e;
-            uint4 w = make_uint4(0u, 0u, 0u, 0u);
-            if (rem > 0) w.x = __ldg(wp);
-            if (rem > 1) w.y = __ldg(wp + G);
-            if (rem > 2) w.z = __ldg(wp + 2 * G);
-            if (rem > 3) w.w = __ldg(wp + 3 * G);
-            return w;
+            return make_uint4(__ldg(wp), __ldg(wp + G), __ldg(wp + 2 * G), __ldg(wp + 3 * G));
         };
         int4 me = meta_at(sl), mn = meta_at(sl + G);
-        uint4 wn = words_at(me.x, me.y);
+        uint4 wn = words_at(me.x);
 #pragma unroll 1
-        for (int p = sl; p < nnz; p += G) {
+        for (int p = sl; p - sl < nnz; p += G) {
             float *ap = reinterpret_cast<float *>(sm.A) + me.z;
             const float av = *ap, fac = mh * __int_as_float(me.w);
-            int e = me.x, rem = me.y;
+            int e = me.x, rem = me.y, chunks = (__shfl_sync(kFull, rem, 0) + 3) >> 2;
             uint4 w = wn;
             me = mn;
             mn = meta_at(p + 2 * G);
-            wn = words_at(me.x, me.y);
             float a0 = 0.f, a1 = 0.f;
 #pragma unroll 1
-            for (;;) {
-                // (a missing term's word is 0: D entry 0 is read and not used)
-                const float v0 = Dv[w.x & 0x7fffffu], v1 = Dv[w.y & 0x7fffffu], v2 = Dv[w.z & 0x7fffffu],
-                            v3 = Dv[w.w & 0x7fffffu];
-                const uint4 wc = w;
-                const int rc = rem;
+            do {
+                const unsigned x0 = rem > 0 ? w.x : 0u, x1 = rem > 1 ? w.y : 0u, x2 = rem > 2 ? w.z : 0u,
+                               x3 = rem > 3 ? w.w : 0u;
+                const bool whole = rem > 3;
+                const float v0 = Dv[x0 & 0x7fffffu], v1 = Dv[x1 & 0x7fffffu], v2 = Dv[x2 & 0x7fffffu],
+                            v3 = Dv[x3 & 0x7fffffu];
                 rem -= 4;
                 e += 4 * G;
-                w = words_at(e, rem);
-                if (rc >= 4) {
-                    a0 = fmaf(coef(wc.x), v0, a0);
-                    a1 = fmaf(coef(wc.y), v1, a1);
-                    a0 = fmaf(coef(wc.z), v2, a0);
-                    a1 = fmaf(coef(wc.w), v3, a1);
-                } else {
-                    a0 = fmaf(coef(wc.x), v0, a0);
-                    if (rc > 1) a0 = fmaf(coef(wc.y), v1, a0);
-                    if (rc > 2) a0 = fmaf(coef(wc.z), v2, a0);
-                }
-                if (rem <= 0) break;
-            }
-            *ap = fmaf(fac, a0 + a1, av);
+                --chunks;
+                w = words_at(chunks > 0 ? e : me.x);
+                a0 = fmaf(coef(x0), v0, a0);
+                const float b = fmaf(coef(x1), v1, whole ? a1 : a0);
+                a0 = fmaf(coef(x2), v2, whole ? a0 : b);
+                a1 = whole ? fmaf(coef(x3), v3, b) : a1;
+            } while (chunks > 0);
+            wn = w;
+            if (p < nnz) *ap = fmaf(fac, a0 + a1, av);
         }
         __syncwarp();
     } else {
