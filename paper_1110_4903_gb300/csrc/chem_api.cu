@@ -827,16 +827,30 @@ int launch_cfg(Handle *h, const chem_advance_args *a, int prec, const LaunchCfg 
     const long long cells_per_warp = 32 / cfg->G;
     const long long warps = (b.n_cells + cells_per_warp - 1) / cells_per_warp;
     int wpb = cfg->block / 32;
+    long long blocks_per_sm = cfg->grid / h->num_sms;
     if (warps < (long long)cfg->grid * wpb) {
         const long long per_sm = (warps + h->num_sms - 1) / h->num_sms;
-        const long long blocks_per_sm = (per_sm + wpb - 1) / wpb;
+        blocks_per_sm = (per_sm + wpb - 1) / wpb;
         wpb = (int)((per_sm + blocks_per_sm - 1) / blocks_per_sm);
     }
     const size_t smem =
         (size_t)(kBlockHeaderBytes + wpb * cells_per_warp * slot_stride(h->mech, prec == CHEM_MIXED ? 4 : 8, cfg->G));
     const long long grid = std::min<long long>(cfg->grid, (warps + wpb - 1) / wpb);
     void *args[] = {&h->mech, &o, &b};
-    e = cudaLaunchKernel(cfg->fn, dim3((unsigned)grid), dim3((unsigned)wpb * 32), args, smem, st);
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3((unsigned)grid);
+    lc.blockDim = dim3((unsigned)wpb * 32);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    // what the blocks do not need of the SM's shared memory serves as L1
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    const long long sm_smem = h->max_smem_optin + 1024;
+    at.val.sharedMemCarveout =
+        (unsigned)std::min<long long>(100, (100 * blocks_per_sm * ((long long)smem + 1024) + sm_smem - 1) / sm_smem);
+    lc.attrs = &at;
+    lc.numAttrs = 1;
+    e = cudaLaunchKernelExC(&lc, cfg->fn, args);
     if (e != cudaSuccess) return cuda_fail(e, "launching the step kernel");
     h->launches.fetch_add(1);
     return CHEM_OK;
