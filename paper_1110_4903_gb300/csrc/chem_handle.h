@@ -66,8 +66,15 @@ int get_cfg(Handle *h, int prec, int G, LaunchCfg **out, bool queue = false);
 int configure(Handle *h, int prec, int G, int wpb, LaunchCfg &cfg, bool queue = false);
 const void *be_kernel_queue(int prec, int G);
 int launch_step(Handle *h, const chem_advance_args *a, int prec, int G, unsigned long long *counter);
+// A launch that is one of a chain over parts of one step (segments): the
+// parts touch different cells, so that each may start while the one before
+// it still runs.  The counters of a chain are zeroed before its first launch.
+struct LaunchChain {
+    bool first = true, last = true;   // of its chain
+    int max_wpb = 0;                  // warps per block at most (0: the shape's own)
+};
 int launch_cfg(Handle *h, const chem_advance_args *a, int prec, const LaunchCfg *cfg,
-               unsigned long long *counter);
+               unsigned long long *counter, const LaunchChain *chain = nullptr);
 unsigned long long *next_counter(Handle *h);
 StepOptions step_options(const Handle *h, int prec);
 void fill_log_table(std::vector<double> &tab);

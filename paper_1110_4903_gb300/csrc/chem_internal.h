@@ -232,6 +232,9 @@ struct StepBatch {
     int *substeps;
     int *failures;
     unsigned long long *work_counter;   // zeroed before the launch
+    // one launch of a chain over parts of a step: the next may start once
+    // every block of this one runs; this one ends after the one before it
+    int chain_next, chain_prev;
     // optional record of the substep schedule: kSchedWords words per cell,
     // bit a set when attempt a was accepted (the attempt budget is capped at
     // 32 kSchedWords while recording)

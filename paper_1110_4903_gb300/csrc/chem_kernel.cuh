@@ -1613,6 +1613,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
     SlotMem<JT> sm;
     sm.carve(smem + (size_t)(warp * S + slot) * sbytes, m);
     __syncthreads();
+    if (!Q && b.chain_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     int state = kFree;
     long long cell = -1;
@@ -1895,6 +1896,9 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
         }
         __syncwarp();
     }
+    // (a chain's launches end in order: what follows the last one in its
+    // stream finds all of them done)
+    if (!Q && b.chain_prev) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace chem
