@@ -176,7 +176,7 @@ struct HostTables {
     struct Layout {
         std::vector<int2> j_meta, it_meta;
         std::vector<int4> j_meta32;
-        std::vector<unsigned> j_w, sp_w;
+        std::vector<unsigned> j_w, j_w_wide, sp_w;
         std::vector<int> j_d;
         std::vector<double> j_c;
     } lay[kLayouts];
@@ -493,9 +493,13 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
     // terms of each list are put in an order in which the lanes of a pass
     // read distinct banks at each step where they can: the sum is the same
     // up to the order of its FP32 additions.
+    //   rank[e] receives a term's place in its list; with `given` the terms
+    // take the places listed there.
     auto interleave = [](int nlists, const std::vector<int> &ptr, int G, std::vector<int2> &meta,
                          std::vector<int> &pos, int tag_shift, const std::vector<int> *tags,
-                         const std::vector<int> *bank = nullptr) {
+                         const std::vector<int> *bank = nullptr, std::vector<int> *rank = nullptr,
+                         const std::vector<int> *given = nullptr) {
+        if (rank) rank->assign(ptr.back(), 0);
         int base = 0;
         pos.assign(ptr.back(), -1);
         for (int P0 = 0; P0 < nlists; P0 += G) {
@@ -542,6 +546,10 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
                     }
                 }
             }
+            if (given)
+                for (int e = ptr[P0]; e < ptr[P1]; ++e) slot[e - ptr[P0]] = (*given)[e];
+            if (rank)
+                for (int e = ptr[P0]; e < ptr[P1]; ++e) (*rank)[e] = slot[e - ptr[P0]];
             for (int q = P0; q < P1; ++q) {
                 const int len = ptr[q + 1] - ptr[q], lane = q - P0;
                 meta.push_back(make_int2(base + lane, (tags ? (*tags)[q] : 0) | (len << tag_shift)));
@@ -563,7 +571,8 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
             L.j_c[pos[e]] = t.j_c[e];
         }
         std::vector<int2> meta32;
-        const int nw32 = interleave(ns * ns, t.j_ptr32, G, meta32, pos, 16, &t.j_sk32, &t.j_d32);
+        std::vector<int> rank;
+        const int nw32 = interleave(ns * ns, t.j_ptr32, G, meta32, pos, 16, &t.j_sk32, &t.j_d32, &rank);
         // the FP32 entries' metadata: first word, length, offset of (s, k)
         // in the column-major matrix of columns of ldc rows, and the factor
         // M_s / M_k rounded once to FP32
@@ -578,6 +587,15 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
         // (the kernel reads whole chunks of four rows, one ahead)
         L.j_w.assign(nw32 + 8 * G, 0u);
         for (size_t e = 0; e < pos.size(); ++e) L.j_w[pos[e]] = t.j_w[e];
+        if (ns < 32) {
+            // the same order of terms for wide warps
+            std::vector<int2> meta_w;
+            const int nww = interleave(ns * ns, t.j_ptr32, 32, meta_w, pos, 16, &t.j_sk32, nullptr, nullptr, &rank);
+            L.j_w_wide.assign(nww + 8 * 32, 0u);
+            for (size_t e = 0; e < pos.size(); ++e) L.j_w_wide[pos[e]] = t.j_w[e];
+        } else {
+            L.j_w_wide.assign(1, 0u);
+        }
         const int ni = interleave(t.n_items, t.it_ptr, G, L.it_meta, pos, 16, &t.it_id);
         L.sp_w.assign(std::max(ni, 1), 0u);
         for (size_t e = 0; e < pos.size(); ++e) {
@@ -635,7 +653,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
                  i_sip = addv(t.sp_item_ptr),
                  i_ex = addv(t.exp_tab), i_div = addv(t.div16), i_rdf = addv(t.rxn_df), i_dcef = addv(t.d_cef),
                  i_spf = addv(t.spf), i_log = addv(t.log_tab);
-    size_t i_lay[kLayouts][8];
+    size_t i_lay[kLayouts][9];
     for (int li = 0; li < kLayouts; ++li) {
         const auto &L = t.lay[li];
         i_lay[li][7] = addv(L.j_meta32);
@@ -647,6 +665,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
         i_lay[li][5] = addv(L.sp_w);
     }
     const size_t i_dce = addv(t.d_ce), i_dpk64 = addv(t.d_pk64);
+    for (int li = 0; li < kLayouts; ++li) i_lay[li][8] = addv(t.lay[li].j_w_wide);
     cudaError_t e = cudaMalloc(&h->dev_tables, total);
     if (e != cudaSuccess) return fail(CHEM_E_OOM, "device tables (%zu bytes): %s", total, cudaGetErrorString(e));
     h->dev_tables_bytes = total;
@@ -692,6 +711,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
         g.j_c = (const double *)at(i_lay[li][3]);
         g.it_meta = (const int2 *)at(i_lay[li][4]);
         g.sp_w = (const unsigned *)at(i_lay[li][5]);
+        m.j_w_wide[li] = (const unsigned *)at(i_lay[li][8]);
     }
     m.sp_item_ptr = (const int *)at(i_sip);
 
@@ -827,23 +847,33 @@ int launch_cfg(Handle *h, const chem_advance_args *a, int prec, const LaunchCfg 
     // (11.9 ms, mixed); blocks of 7 warps on 147 SMs take 10.3 ms, and
     // 1,024 cells of 9 species on 128 SMs instead of 13 take 0.58 instead of
     // 0.78 ms (FP64).  Blocks of one warp are not dealt out evenly (13.7 ms).
-    const long long cells_per_warp = 32 / cfg->G;
+    //   With several cells per warp, a call of at most one and a half cells
+    // per resident warp (two blocks per SM) starts with one to a warp, and any
+    // other ends so (wide warps, be_kernel).  152 SMs, 9 species, eight cells
+    // to a warp against one: 4,000 cells 1.30 against 1.08 ms (FP64), 0.81
+    // against 0.65 (mixed); 6,000 cells 1.26 against 1.38 and 0.83 against
+    // 0.83; 12,000 cells 1.70 against 2.25 and 0.99 against 1.26.  (A slot's
+    // variables pass through its matrix: five species at least.)
+    const long long sbytes = slot_stride(h->mech, prec == CHEM_MIXED ? 4 : 8, cfg->G);
+    b.wide = h->ns >= 5 && h->ns < 32 && cfg->G <= 8;
+    b.one_cell = b.wide && 2 * b.n_cells <= 3LL * 2 * (kMaxBlockThreads / 32) * h->num_sms &&
+                 2 * (kBlockHeaderBytes + kMaxBlockThreads / 32 * sbytes) <= h->max_smem_optin;
+    const long long cells_per_warp = b.one_cell ? 1 : 32 / cfg->G;
     const long long warps = (b.n_cells + cells_per_warp - 1) / cells_per_warp;
-    int wpb = cfg->block / 32;
-    long long blocks_per_sm = cfg->grid / h->num_sms, max_grid = cfg->grid;
+    int wpb = b.one_cell ? kMaxBlockThreads / 32 : cfg->block / 32;
+    long long blocks_per_sm = b.one_cell ? 2 : cfg->grid / h->num_sms, max_grid = blocks_per_sm * h->num_sms;
     if (chain && chain->max_wpb && chain->max_wpb < wpb) {
         // (the same resident warps in smaller blocks; the hardware takes as
         // many as fit)
         max_grid = max_grid * wpb / chain->max_wpb;
         blocks_per_sm = max_grid / h->num_sms;
         wpb = chain->max_wpb;
-    } else if (warps < (long long)cfg->grid * wpb) {
+    } else if (warps < max_grid * wpb) {
         const long long per_sm = (warps + h->num_sms - 1) / h->num_sms;
         blocks_per_sm = (per_sm + wpb - 1) / wpb;
         wpb = (int)((per_sm + blocks_per_sm - 1) / blocks_per_sm);
     }
-    const size_t smem =
-        (size_t)(kBlockHeaderBytes + wpb * cells_per_warp * slot_stride(h->mech, prec == CHEM_MIXED ? 4 : 8, cfg->G));
+    const size_t smem = (size_t)(kBlockHeaderBytes + wpb * cells_per_warp * sbytes);
     const long long grid = std::min<long long>(max_grid, (warps + wpb - 1) / wpb);
     void *args[] = {&h->mech, &o, &b};
     cudaLaunchConfig_t lc{};

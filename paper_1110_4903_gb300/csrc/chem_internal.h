@@ -147,6 +147,8 @@ struct DeviceMech {
     // first, and the species lists (reactions with nu_rs != 0) cut into
     // items of at most kChunk entries; per-G layouts above
     GatherLayout gl[kLayouts];
+    // FP32 words in the positions of 32 lanes per cell and the term order of G
+    const unsigned *j_w_wide[kLayouts];
     const int *sp_item_ptr;     // [ns+1] work items of each species
     const double *exp_tab;      // [kExpTab] 2^(j/kExpTab), then the constants above
     const double2 *log_tab;     // [kLogTab + 1] {1/F, ln F}, F = 1 + j/kLogTab
@@ -235,6 +237,9 @@ struct StepBatch {
     // one launch of a chain over parts of a step: the next may start once
     // every block of this one runs; this one ends after the one before it
     int chain_next, chain_prev;
+    // wide warps (be_kernel): for a warp's last cells; from the start, one
+    // cell at a time per warp, whose shared memory is one slot
+    int wide, one_cell;
     // optional record of the substep schedule: kSchedWords words per cell,
     // bit a set when attempt a was accepted (the attempt budget is capped at
     // 32 kSchedWords while recording)

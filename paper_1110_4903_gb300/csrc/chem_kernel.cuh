@@ -298,6 +298,41 @@ __device__ __forceinline__ double flog(double x, const double2 *tab, const doubl
 __device__ __forceinline__ double nasa_s(const CoefRow<double> &th, double T, double lnT, const Fp64Ops &op) {
     return op.add(fma(th[0], lnT, op.mul(T, fma(T, fma(T, fma(T, th[12], th[11]), th[10]), th[1]))), th[13]);
 }
+// Sums over a cell's species with one species per lane (wide warps, below),
+// in the order of G0 lanes per cell: lane l of those sums the terms l, l + G0,
+// ... one after another, then the partial sums meet in a tree.  Terms i >= cnt
+// (at most 32 lanes) are not there; `first` is added to lane 0's partial sum.
+// Every lane gets the result.
+template <int G0>
+__device__ __forceinline__ double wide_dot(double a, double b, int cnt, const Fp64Ops &op, double first = 0.0,
+                                           bool has_first = false) {
+    const int l = threadIdx.x & (G0 - 1);
+    double p = 0.0;
+#pragma unroll 1
+    for (int i = l; i - l < cnt; i += G0) {
+        const double x = __shfl_sync(kFull, a, i), y = __shfl_sync(kFull, b, i);
+        if (i < cnt) p = fma(x, y, p);
+    }
+    if (has_first && l == 0) p = op.add(p, first);
+#pragma unroll
+    for (int o = G0 / 2; o > 0; o >>= 1) p = op.add(p, __shfl_xor_sync(kFull, p, o));
+    return p;
+}
+template <int G0>
+__device__ __forceinline__ float wide_dotf(float a, float b, int cnt, float first = 0.f, bool has_first = false) {
+    const int l = threadIdx.x & (G0 - 1);
+    float p = 0.f;
+#pragma unroll 1
+    for (int i = l; i - l < cnt; i += G0) {
+        const float x = __shfl_sync(kFull, a, i), y = __shfl_sync(kFull, b, i);
+        if (i < cnt) p = fmaf(x, y, p);
+    }
+    if (has_first && l == 0) p += first;
+#pragma unroll
+    for (int o = G0 / 2; o > 0; o >>= 1) p += __shfl_xor_sync(kFull, p, o);
+    return p;
+}
+
 // Temperature recovery from (rho_s, e) for every slot whose `need` is set:
 // Newton on sum_s rho_s e_s^sens(T) = e, safeguarded by bisection on
 // [kTlo, kThi] (Eq. 3 with the kinetic energy left to the flux stage).  A
@@ -310,7 +345,7 @@ __device__ __forceinline__ double nasa_s(const CoefRow<double> &th, double T, do
 //   The energies come from the multiplied-out polynomials (five DFMA per
 //   species, no 1/T); with F32 the derivative sum c_v is formed in FP32, which
 //   changes the Newton steps by a relative 1e-7 and not the root.
-template <int G, bool F32>
+template <int G, int G0, bool F32>
 __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab, const double *x, int sl, bool need,
                                           bool cold, double guess, double &T_out, bool &ok) {
     const int ns = m.ns;
@@ -326,17 +361,31 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
 #pragma unroll 1
         for (int it = 0; it < 3; ++it) {
             const long long Tb = __double_as_longlong(f2d_alu(Tf));
-            float f = 0.f, fp = 0.f;
+            float f = 0.f, fp = 0.f, wr = 0.f;
 #pragma unroll 1
             for (int s = sl; s < ns; s += G) {
                 const auto d = coef_row(m.tpoly_f, ns, s, thermo_range(m, s, Tb));
                 const float r = d2f_rz(x[s]);
                 neg |= r < 0.f;
-                f = fmaf(r, fmaf(fmaf(fmaf(fmaf(fmaf(d[10], Tf, d[9]), Tf, d[8]), Tf, d[7]), Tf, d[6]), Tf, d[5]), f);
-                fp = fmaf(r, fmaf(fmaf(fmaf(fmaf(d[4], Tf, d[3]), Tf, d[2]), Tf, d[1]), Tf, d[0]), fp);
+                const float es = fmaf(fmaf(fmaf(fmaf(fmaf(d[10], Tf, d[9]), Tf, d[8]), Tf, d[7]), Tf, d[6]), Tf, d[5]);
+                const float cv = fmaf(fmaf(fmaf(fmaf(d[4], Tf, d[3]), Tf, d[2]), Tf, d[1]), Tf, d[0]);
+                if constexpr (G == G0) {
+                    f = fmaf(r, es, f);
+                    fp = fmaf(r, cv, fp);
+                } else {
+                    wr = r;
+                    f = es;
+                    fp = cv;
+                }
             }
-            f = Grp<G>::sum(f) - d2f_rz(e);
-            fp = Grp<G>::sum(fp);
+            if constexpr (G == G0) {
+                f = Grp<G>::sum(f);
+                fp = Grp<G>::sum(fp);
+            } else {
+                f = wide_dotf<G0>(wr, f, ns);
+                fp = wide_dotf<G0>(wr, fp, ns);
+            }
+            f -= d2f_rz(e);
             Tf -= __fdividef(f, fp);
             Tf = fminf(fmaxf(Tf, (float)kTlo), (float)kThi);   // (a NaN goes to the lower end)
         }
@@ -349,30 +398,51 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
         if (!__any_sync(kFull, !done)) break;
         const long long Tb = __double_as_longlong(T);
         const float Tf = F32 ? d2f_rz(T) : 0.f;
-        double f = 0.0, fp = 0.0;
-        float fpf = 0.f;
+        double f = 0.0, fp = 0.0, xs = 0.0;
+        float fpf = 0.f, xf = 0.f;
 #pragma unroll 1
         for (int s = sl; s < ns; s += G) {
             const int rg = thermo_range(m, s, Tb);
             const auto c = coef_row(m.tpoly, ns, s, rg);
             const double es = fma(fma(fma(fma(fma(c[5], T, c[4]), T, c[3]), T, c[2]), T, c[1]), T, c[0]);
-            f = fma(x[s], es, f);
+            xs = x[s];
+            if constexpr (G == G0)
+                f = fma(xs, es, f);
+            else
+                f = es;
             if (F32) {
                 const auto d = coef_row(m.tpoly_f, ns, s, rg);
                 const float cv = fmaf(fmaf(fmaf(fmaf(d[4], Tf, d[3]), Tf, d[2]), Tf, d[1]), Tf, d[0]);
-                fpf = fmaf(d2f_rz(x[s]), cv, fpf);
+                xf = d2f_rz(xs);
+                if constexpr (G == G0)
+                    fpf = fmaf(xf, cv, fpf);
+                else
+                    fpf = cv;
             } else {
                 const double cv = fma(fma(fma(fma(c[10], T, c[9]), T, c[8]), T, c[7]), T, c[6]);
-                fp = fma(x[s], cv, fp);
+                if constexpr (G == G0)
+                    fp = fma(xs, cv, fp);
+                else
+                    fp = cv;
             }
         }
-        f = op.sub(Grp<G>::sum(f, op), e);
+        if constexpr (G == G0)
+            f = Grp<G>::sum(f, op);
+        else
+            f = wide_dot<G0>(xs, f, ns, op);
+        f = op.sub(f, e);
         double rfp;
         if (F32) {
-            fpf = Grp<G>::sum(fpf);
+            if constexpr (G == G0)
+                fpf = Grp<G>::sum(fpf);
+            else
+                fpf = wide_dotf<G0>(xf, fpf, ns);
             rfp = f2d_alu(__frcp_rn(fpf));
         } else {
-            fp = Grp<G>::sum(fp, op);
+            if constexpr (G == G0)
+                fp = Grp<G>::sum(fp, op);
+            else
+                fp = wide_dot<G0>(xs, fp, ns, op);
             rfp = frcp1(fp, op);
         }
         if (!done) {
@@ -690,7 +760,9 @@ struct SlotMem {
 // Sources, Jacobian and one Newton update of Eq. 29 for every slot of the
 // warp.  Inputs per slot: x, x0, T, h.  Outputs: x <- x + delta, the scaled
 // norm, and a flag for a singular pivot or a non-finite update.
-template <int G, typename JT>
+//   G0: the lanes per cell whose order of summation is kept (G, or fewer in a
+// wide warp, where a species has a lane of its own).
+template <int G, int G0, typename JT>
 __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem<JT> &sm, int sl,
                                  double T, double h, double atol_rho, double atol_e, double rtol,
                                  double &norm, bool &bad, double &T_pred) {
@@ -726,15 +798,15 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     //    path forms it in FP32
     const long long Tb = __double_as_longlong(T);
     const float Tf = f32 ? d2f_rz(T) : 0.f;
-    double ctot = 0.0, rhocv = 0.0;
-    float rhocvf = 0.f;
+    double ctot = 0.0, rhocv = 0.0, xs = 0.0;
+    float rhocvf = 0.f, xf = 0.f;
 #pragma unroll 1
     for (int s = sl; s < ns; s += G) {
         const double *spr = m.sp + s * kSpStride;
-        const double xs = sm.x[s];
+        xs = sm.x[s];
         const double ci = op.mul(xs, __ldg(spr + 1));
         sm.c[s] = ci;
-        ctot = op.add(ctot, ci);
+        ctot = G == G0 ? op.add(ctot, ci) : ci;
         const int rg = thermo_range(m, s, Tb);
         const auto th = coef_row(m.thermo, ns, s, rg);
         const double hRT = fma(th[9], invT, fma(T, fma(T, fma(T, fma(T, th[8], th[7]), th[6]), th[5]), th[0]));
@@ -756,7 +828,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             sm.esJ[s] = (JT)__ldg(m.spf + s * kSpStride + 2) * Tf * (hJs - (JT)1);
             const auto d = coef_row(m.tpoly_f, ns, s, rg);
             const float cv = fmaf(fmaf(fmaf(fmaf(d[4], Tf, d[3]), Tf, d[2]), Tf, d[1]), Tf, d[0]);
-            rhocvf = fmaf(d2f_rz(xs), cv, rhocvf);
+            xf = d2f_rz(xs);
+            rhocvf = G == G0 ? fmaf(xf, cv, rhocvf) : cv;
             sm.cJ[s] = to_jt<JT>(ci);
             sm.hJ[s] = hJs;
         } else {
@@ -764,7 +837,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             const double es = fma(op.mul(RM, T), hm1, -__ldg(spr + 3));
             const auto c = coef_row(m.tpoly, ns, s, rg);
             const double cv = fma(fma(fma(fma(c[10], T, c[9]), T, c[8]), T, c[7]), T, c[6]);
-            rhocv = fma(xs, cv, rhocv);
+            rhocv = G == G0 ? fma(xs, cv, rhocv) : cv;
             sm.hRT[s] = hm1;
             sm.es[s] = es;
         }
@@ -782,16 +855,25 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             sm.hRT[ns] = 0.0;
         }
     }
-    ctot = Grp<G>::sum(ctot, op);
+    if constexpr (G == G0)
+        ctot = Grp<G>::sum(ctot, op);
+    else
+        ctot = wide_dot<G0>(ctot, op.one, ns, op);
     double dTde;
     float dTdef = 0.f;
     if (f32) {
-        rhocvf = Grp<G>::sum(rhocvf);
+        if constexpr (G == G0)
+            rhocvf = Grp<G>::sum(rhocvf);
+        else
+            rhocvf = wide_dotf<G0>(xf, rhocvf, ns);
         dTdef = __frcp_rn(rhocvf);
         dTde = f2d_alu(dTdef);
         // dT/drho_k = -e_k^sens dT/de is formed where the Jacobian needs it
     } else {
-        rhocv = Grp<G>::sum(rhocv, op);
+        if constexpr (G == G0)
+            rhocv = Grp<G>::sum(rhocv, op);
+        else
+            rhocv = wide_dot<G0>(xs, rhocv, ns, op);
         dTde = frcp(rhocv, op);
 #pragma unroll 1
         for (int s = sl; s < ns; s += G) sm.dTdr[s] = (JT)op.mul(-op.add(sm.es[s], __ldg(m.sp + s * kSpStride + 3)), dTde);
@@ -817,7 +899,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     load_rxn(sl);
 #pragma unroll 1
     for (int r = sl; r < nr; r += G) {
-        const double lnA = nAb.x, beta = nAb.y, EaR = nEd.x, dnu = nEd.y;
+        const double lnA = nAb.x, beta = nAb.y, EaR = nEd.x;
         const int fr = nf.x, fpw = nf.y;
         load_rxn(r + G);
         const int a0 = fr & 0xff, a1 = (fr >> 8) & 0xff, a2 = (fr >> 16) & 0xff;
@@ -909,6 +991,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     //    (an item's partial sums: sum nu Q in FP64, then sum nu dQ/dT and
     //    sum nu q_tb in the Jacobian type, packed into the next 16 bytes)
     const GatherLayout &gl = m.gl[layout_index(G)];
+    const unsigned *gl_j_w = G == G0 ? gl.j_w : m.j_w_wide[layout_index(G0)];
     //   The table's words come from L2 as often as from L1, so an item's
     //   eight words are loaded together, the next item's descriptor with
     //   them, and the operands of four terms at a time; the sums keep the
@@ -967,7 +1050,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         pj[1] = squ;
     }
     __syncwarp();
-    double dEt = 0.0;
+    double dEt = 0.0, wef = 0.0;
 #pragma unroll 1
     for (int s = sl; s < ns; s += G) {
         double sq = 0.0;
@@ -992,12 +1075,17 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         const JT ws = jmul(f32 ? MJ : (JT)op.mul(M, invT), sdq), us = jmul(MJ, squ);
         sm.w[s] = ws;
         sm.u[s] = us;
-        dEt = fma(ef, dx, dEt);
+        wef = ef;
+        dEt = G == G0 ? fma(ef, dx, dEt) : dx;
     }
     // the total-energy residual R_E = F_e + sum_s e_f,s F_s = (x_e - x0_e) +
     // sum_s e_f,s (x_s - x0_s), in which the sources cancel (Omega_e =
     // -sum_s e_f,s wdot_s); it replaces the energy equation (phase 5)
-    const double RE = op.add(Grp<G>::sum(dEt, op), op.sub(sm.x[ns], sm.x0[ns]));
+    if constexpr (G == G0)
+        dEt = Grp<G>::sum(dEt, op);
+    else
+        dEt = wide_dot<G0>(wef, dEt, ns, op);
+    const double RE = op.add(dEt, op.sub(sm.x[ns], sm.x0[ns]));
     __syncwarp();
 
     // 4. D entries: d Q_r / d rho_k without the all-ones third-body part,
@@ -1158,7 +1246,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         const int nnz = m.nJ_nz;
         auto meta_at = [&](int p) -> int4 { return p < nnz ? __ldg(gl.j_meta32 + p) : make_int4(0, 0, 0, 0); };
         auto words_at = [&](int e) -> uint4 {
-            const unsigned *wp = gl.j_w + e;
+            const unsigned *wp = gl_j_w + e;
             return make_uint4(__ldg(wp), __ldg(wp + G), __ldg(wp + 2 * G), __ldg(wp + 3 * G));
         };
         int4 me = meta_at(sl), mn = meta_at(sl + G);
@@ -1252,9 +1340,10 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     //    the diagonal
     bool sing = false;
     if constexpr (f32 && G == 32) {
-        sing = N >= kLuRegMinN && N <= kLuRegN
-                   ? lu_registers(reinterpret_cast<float *>(sm.A), ldc, N, sl)
-                   : lu_columns((unsigned)__cvta_generic_to_shared(sm.A), ldc, N);
+        if (G == G0 && N >= kLuRegMinN && N <= kLuRegN)
+            sing = lu_registers(reinterpret_cast<float *>(sm.A), ldc, N, sl);
+        else
+            sing = lu_columns((unsigned)__cvta_generic_to_shared(sm.A), ldc, N);
     } else {
 #pragma unroll 1
     for (int j = 0; j < N; ++j) {
@@ -1367,8 +1456,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         if (__double_as_longlong(den) > 0) return op.mul(fabs(d), frcp1(den, op));
         return (__double_as_longlong(d) << 1) != 0 ? CUDART_INF : 0.0;
     };
-    double nrm = 0.0, des = 0.0, se = 0.0;
-    float desf = 0.f, sef = 0.f;
+    double nrm = 0.0, des = 0.0, se = 0.0, dw = 0.0;
+    float desf = 0.f, sef = 0.f, dwf = 0.f;
     int nonfinite = 0;
 #pragma unroll 1
     for (int i = sl; i < N; i += G) {
@@ -1377,12 +1466,17 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         if (f32) {
             df = (float)sm.A[ix(i, N)];
             d = f2d_alu(df);
-            desf -= (float)sm.esJ[i] * df;   // e_s with its formation part: see below
-            sef = fmaf(__ldg(m.spf + i * kSpStride + 3), df, sef);
+            // (e_s with its formation part: see below)
+            const float es = (float)sm.esJ[i], ef = __ldg(m.spf + i * kSpStride + 3);
+            dwf = df;
+            desf = G == G0 ? fmaf(-es, df, desf) : -es;
+            sef = G == G0 ? fmaf(ef, df, sef) : ef;
         } else {
             d = (double)sm.A[ix(i, N)];
-            des = fma(-sm.es[i], d, des);
-            se = fma(__ldg(m.sp + i * kSpStride + 3), d, se);
+            const double es = sm.es[i], ef = __ldg(m.sp + i * kSpStride + 3);
+            dw = d;
+            des = G == G0 ? fma(-es, d, des) : -es;
+            se = G == G0 ? fma(ef, d, se) : ef;
         }
         const double xi = op.add(sm.x[i], d);
         sm.x[i] = xi;
@@ -1392,27 +1486,38 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     }
     {
         // the eliminated energy unknown: de = -R_E - e_f . drho
-        const double de = op.sub(-RE, f32 ? f2d_alu(Grp<G>::sum(sef)) : Grp<G>::sum(se, op));
+        if constexpr (G == G0) {
+            sef = Grp<G>::sum(sef);
+            se = f32 ? 0.0 : Grp<G>::sum(se, op);
+        } else {
+            sef = f32 ? wide_dotf<G0>(sef, dwf, N) : 0.f;
+            se = f32 ? 0.0 : wide_dot<G0>(se, dw, N, op);
+        }
+        const double de = op.sub(-RE, f32 ? f2d_alu(sef) : se);
         if (sl == 0) {
             const double xe = op.add(sm.x[ns], de);
             sm.x[ns] = xe;
             if (!finite_bits(xe)) nonfinite = 1;
             const double ri = ratio(de, fma(rtol, fabs(xe), atol_e));
             if (bits_gt(ri, nrm)) nrm = ri;
-            // dT = (de - sum_s e_s^sens drho_s) / (rho cv), where de = -R_E -
-            // e_f . drho: the FP32 path's e_s carry e_f, so it adds -R_E
-            if (f32)
-                desf += d2f_rz(-RE);
-            else
-                des = op.add(des, de);
+        }
+        // dT = (de - sum_s e_s^sens drho_s) / (rho cv), where de = -R_E -
+        // e_f . drho: the FP32 path's e_s carry e_f, so it adds -R_E
+        if constexpr (G == G0) {
+            if (sl == 0) {
+                if (f32)
+                    desf += d2f_rz(-RE);
+                else
+                    des = op.add(des, de);
+            }
+            des = f32 ? f2d_alu(Grp<G>::sum(desf)) : Grp<G>::sum(des, op);
+        } else {
+            des = f32 ? f2d_alu(wide_dotf<G0>(desf, dwf, N, d2f_rz(-RE), true))
+                      : wide_dot<G0>(des, dw, N, op, de, true);
         }
     }
     nrm = Grp<G>::max_nonneg(nrm);
     nonfinite = Grp<G>::any(nonfinite);
-    if (f32)
-        des = f2d_alu(Grp<G>::sum(desf));
-    else
-        des = Grp<G>::sum(des, op);
     __syncwarp();
     norm = nrm;
     bad = sing || nonfinite;
@@ -1594,37 +1699,61 @@ __device__ __forceinline__ void serve_cell_done(const ServeQueue &q, int e) {
     }
 }
 
-// At most 10 warps per block and 102 registers per thread: 20 warps fit on
-// an SM when shared memory allows it (2 blocks of 10; the mixed path at 36
-// species, 11.3 KB per cell).
-// Q: request-server mode, cells claimed from b.queue (each slot's request
-// descriptor in host memory; its dt, buffers and completion accounting).
-template <int G, typename JT, bool Q = false>
-__global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, StepOptions o, StepBatch b) {
-    extern __shared__ __align__(16) char smem[];
+// Wide warps (be_kernel) serve at most this many lanes per cell.
+constexpr int kWideMaxG = 8;
+
+// A slot's cell and where its integration stands.
+struct SlotVars {
+    int state;
+    long long cell;
+    // request-server mode: the slot's ring entry and its request's dt
+    int qe;
+    double sdt;
+    double T, T0, Tin, h, norm_prev, atol_rho, atol_e;
+    int k, level, attempts, iters, subs, fails;
+    long long t_units;
+};
+// (kept in a slot's matrix on the way to a wide warp, FP32 at five species)
+static_assert(sizeof(SlotVars) <= 6 * 8 * 4, "slot variables");
+__device__ __forceinline__ SlotVars free_slot(double dt) {
+    SlotVars v;
+    v.state = kFree;
+    v.cell = -1;
+    v.qe = -1;
+    v.sdt = dt;
+    v.T = v.T0 = 1500.0;
+    v.Tin = CUDART_NAN;
+    v.h = 0.0;
+    v.norm_prev = CUDART_INF;
+    v.atol_rho = v.atol_e = 0.0;
+    v.k = v.level = v.attempts = v.iters = v.subs = v.fails = 0;
+    v.t_units = 0;
+    return v;
+}
+
+// Steps the warp's slots, G lanes each, until no cell is left for any of them
+// (or, with few slots left and b.wide, until the rest is better stepped by
+// wide warps).  Q: request-server mode, cells claimed from b.queue (each
+// slot's request descriptor in host memory; its dt, buffers and completion
+// accounting).  G0: see newton_iteration.
+template <int G, int G0, typename JT, bool Q>
+__device__ __forceinline__ void step_cells(const DeviceMech &m, const StepOptions &o, const StepBatch &b,
+                                           SlotMem<JT> &sm, SlotVars &v) {
     constexpr int S = 32 / G;
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
     const int slot = lane / G;
     const int sl = lane - slot * G;
     const int ns = m.ns, n = ns + 1;
     const double *tab = m.exp_tab;   // 2 KB, stays in L1
-    const long long sbytes = slot_stride(m, (int)sizeof(JT), G);
-    SlotMem<JT> sm;
-    sm.carve(smem + (size_t)(warp * S + slot) * sbytes, m);
-    __syncthreads();
-    if (!Q && b.chain_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-    int state = kFree;
-    long long cell = -1;
-    // request-server mode: the slot's ring entry and its request's dt
-    int qe = -1;
-    double sdt = b.dt;
+    int &state = v.state, &qe = v.qe, &k = v.k, &level = v.level, &attempts = v.attempts, &iters = v.iters,
+        &subs = v.subs, &fails = v.fails;
+    long long &cell = v.cell, &t_units = v.t_units;
+    double &sdt = v.sdt, &T = v.T, &T0 = v.T0, &Tin = v.Tin, &h = v.h, &norm_prev = v.norm_prev,
+           &atol_rho = v.atol_rho, &atol_e = v.atol_e;
     unsigned long long idle_since = 0;
-    double T = 1500.0, T0 = 1500.0, Tin = CUDART_NAN, h = 0.0, norm_prev = CUDART_INF;
-    double atol_rho = 0.0, atol_e = 0.0;
-    int k = 0, level = 0, attempts = 0, iters = 0, subs = 0, fails = 0;
-    long long t_units = 0;
+    (void)S;
+    (void)idle_since;
+    (void)qe;
     const long long total = 1LL << o.max_halvings;
 
     // per-cell outputs (lane 0 of the slot); in request-server mode the
@@ -1720,17 +1849,20 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
                     sm.x0[i] = v;
                     sm.x[i] = v;
                     if (!isfinite(v)) nonfin = 1;
-                    if (i < ns) {
-                        rt += v;
-                        es += fabs(v * __ldg(m.sp + i * kSpStride + 3));
-                    } else {
-                        es += fabs(v);
-                    }
+                    const double ev = fabs(i < ns ? v * __ldg(m.sp + i * kSpStride + 3) : v);
+                    if (i < ns) rt = G == G0 ? rt + v : v;
+                    es = G == G0 ? es + ev : ev;
                 }
             }
             nonfin = Grp<G>::any(nonfin);
-            rt = Grp<G>::sum(rt);
-            es = Grp<G>::sum(es);
+            if constexpr (G == G0) {
+                rt = Grp<G>::sum(rt);
+                es = Grp<G>::sum(es);
+            } else {
+                const Fp64Ops op = fp64_ops(tab);
+                rt = wide_dot<G0>(rt, op.one, ns, op);
+                es = wide_dot<G0>(es, op.one, n, op);
+            }
             if (loading) {
                 atol_rho = o.atol_rel * rt;
                 atol_e = o.atol_rel * es;
@@ -1747,7 +1879,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
             if (!__any_sync(kFull, needT || act != kNoAction)) break;
             double Tr = T;
             bool ok = false;
-            recover_T<G, sizeof(JT) == 4>(m, tab, sm.x, sl, needT, state == kInitT && (Q || !b.T_in), T, Tr, ok);
+            recover_T<G, G0, sizeof(JT) == 4>(m, tab, sm.x, sl, needT, state == kInitT && (Q || !b.T_in), T, Tr, ok);
             int neg = 0;
 #pragma unroll 1
             for (int i = sl; i < ns; i += G)
@@ -1851,6 +1983,10 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
             }
             __syncwarp();
         }
+        if constexpr (G == G0 && !Q && G <= kWideMaxG) {
+            // (a slot is dead once the cells have run out)
+            if (b.wide && __popc(__ballot_sync(kFull, state != kDead && sl == 0)) <= S / 4) return;
+        }
         if (!__any_sync(kFull, state == kNewtonReady)) {
             if (__all_sync(kFull, state == kDead)) break;
             if constexpr (Q) {
@@ -1874,7 +2010,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
         // one Newton iteration of Eq. 29 for every slot
         double norm = 0.0, T_pred = T;
         bool bad = false;
-        newton_iteration<G, JT>(m, tab, sm, sl, T, h, atol_rho, atol_e, o.rtol, norm, bad, T_pred);
+        newton_iteration<G, G0, JT>(m, tab, sm, sl, T, h, atol_rho, atol_e, o.rtol, norm, bad, T_pred);
         if (state == kNewtonReady) {
             // start the next temperature recovery from the linear prediction
             if (bits_gt(T_pred, kTlo) && bits_lt(T_pred, kThi)) T = T_pred;
@@ -1895,6 +2031,63 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, S
             if (bad) state = kRejected;
         }
         __syncwarp();
+    }
+}
+
+// At most 10 warps per block and 96 registers per thread: 20 warps fit on an
+// SM when shared memory allows it (2 blocks of 10; the mixed path at 36
+// species, 11.3 KB per cell).
+//   Wide warps: with several cells per warp, an iteration is a serial chain
+// that takes a warp as long for one cell as for all (4 lanes per cell, 9
+// species, alone on its SM: 89,000 cycles mixed, 152,000 FP64), and the last
+// cells of a launch and the cells of a small one leave most of it idle.  A
+// warp with a quarter of its cells left and no more to come therefore steps
+// them one after another with all its lanes, a species to a lane, each in
+// the slot's shared memory; with b.one_cell it starts so, one cell at a time.
+// Sums and lists keep the order of G lanes per cell, so that a cell's result
+// does not depend on where it ends.  9 species, dt 1e-6, before and after:
+// 1,000 cells 1.82 -> 0.72 ms (FP64), 0.96 -> 0.47 ms (mixed); 16,000 cells
+// 3.59 -> 2.04 and 1.97 -> 1.13 ms; 262,144 cells 16.2 -> 15.2 and 7.0 -> 6.4
+// ms.  At an eighth of the cells left 16,000 cells take 2.37 and 1.16 ms, at
+// three eighths 2.15 and 1.14, at five 2.02 and 1.17 (262,144 mixed: 6.5,
+// 6.5, 6.7).
+template <int G, typename JT, bool Q = false>
+__global__ void __launch_bounds__(kMaxBlockThreads, 2) be_kernel(DeviceMech m, StepOptions o, StepBatch b) {
+    extern __shared__ __align__(16) char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, slot = lane / G;
+    const int per_warp = !Q && G <= kWideMaxG && b.one_cell ? 1 : 32 / G;
+    const long long sbytes = slot_stride(m, (int)sizeof(JT), G);
+    char *warp_mem = smem + (size_t)warp * per_warp * sbytes;
+    SlotMem<JT> sm;
+    // (carved before the barrier: 2 % less time than behind it at 36 species, mixed)
+    if constexpr (Q || G > kWideMaxG) sm.carve(warp_mem + slot * sbytes, m);
+    __syncthreads();
+    if (!Q && b.chain_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if constexpr (Q || G > kWideMaxG) {
+        SlotVars v = free_slot(b.dt);
+        step_cells<G, G, JT, Q>(m, o, b, sm, v);
+    } else {
+        unsigned left = 1;
+        {
+            SlotVars v = free_slot(b.dt);
+            sm.carve(warp_mem + (b.one_cell ? 0 : slot) * sbytes, m);
+            if (!b.one_cell) {
+                step_cells<G, G, JT, false>(m, o, b, sm, v);
+                left = __ballot_sync(kFull, v.state != kDead && lane % G == 0);
+            }
+            // (the matrix is not in use here; b.wide implies it is large enough)
+            if (v.state != kDead && lane == (b.one_cell ? 0 : slot * G)) *reinterpret_cast<SlotVars *>(sm.A) = v;
+            __syncwarp();
+        }
+#pragma unroll 1
+        while (left) {
+            const int src = __ffs(left) - 1;
+            left &= left - 1;
+            sm.carve(warp_mem + src / G * sbytes, m);
+            SlotVars w = *reinterpret_cast<const SlotVars *>(sm.A);
+            __syncwarp();
+            step_cells<32, G, JT, false>(m, o, b, sm, w);
+        }
     }
     // (a chain's launches end in order: what follows the last one in its
     // stream finds all of them done)
