@@ -199,11 +199,8 @@ void fill_log_table(std::vector<double> &tab) {
 void fill_exp_table(std::vector<double> &tab) {
     tab.resize(kExpTabSize);
     for (int j = 0; j < kExpTab; ++j) tab[j] = (double)std::exp2l((long double)j / kExpTab);
-    const double c[kExpTabSize - kExpTab] = {1.0, -0.0,
-                                             369.3299304675746, 6755399441055744.0,
-                                             -0x1.62e42fefa0000p-9, -0x1.cf79abc9e3b3ap-48,
-                                             1.0 / 24.0, 1.0 / 6.0, 0.5, 1.0,
-                                             -1.0 / 6.0, 0.2, -0.25, 1.0 / 3.0, -0.5, 0.6931471805599453};
+    const double c[kExpTabSize - kExpTab] = {1.0, -0.0, -0x1.62e42fefa39efp-9, 0.5,
+                                             1.0 / 3.0, -0.5, 0.6931471805599453, 0.0};
     std::copy(c, c + (kExpTabSize - kExpTab), tab.begin() + kExpTab);
 }
 

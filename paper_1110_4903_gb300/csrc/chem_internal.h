@@ -69,10 +69,10 @@ constexpr int kMaxBlockThreads = 320;
 // Entries of the exp table (2^(j/kExpTab)).
 constexpr int kExpTab = 256;
 // FP64 constants that follow the exp table (the kernels take them as register
-// operands): 1, -0; 256/ln2, 1.5 * 2^52, -ln2/256 in two parts, 1/24, 1/6,
-// 1/2, 1 (the exponential); -1/6, 1/5, -1/4, 1/3, -1/2, ln 2 (the logarithm).
-constexpr int kConstOne = kExpTab, kConstExp = kExpTab + 2, kConstLog = kExpTab + 10;
-constexpr int kExpTabSize = kExpTab + 16;
+// operands): 1, -0; -ln2/256, 1/2 (the exponential); 1/3, -1/2, ln 2 (the
+// logarithm).
+constexpr int kConstOne = kExpTab, kConstExp = kExpTab + 2, kConstLog = kExpTab + 4;
+constexpr int kExpTabSize = kExpTab + 8;
 // Intervals of the log table: kLogTab + 1 entries {1/F, ln F}, F = 1 + j/kLogTab.
 constexpr int kLogTab = 128;
 

@@ -200,24 +200,33 @@ __device__ __forceinline__ double small_pos_int_to_double(int v) {
 }
 
 // exp by the table-driven reduction of P. T. P. Tang, ACM TOMS 15(2), 1989:
-// x = (256 k + j) ln2/256 + r with |r| <= ln2/512, exp(x) = 2^k 2^(j/256) e^r,
-// 2^(j/256) from a 256-entry table and e^r - 1 by its degree-4 Taylor
-// polynomial (truncation below 4e-17 on that interval): eight FP64
-// operations (the integer n = 256 k + j becomes a double on the integer
-// pipe).  exp_reduced: y 2^(n >> 8) = exp(x) for |x| < 2^22, n below 2^31.
-__device__ __forceinline__ double exp_reduced(double x, const double *tab, const Fp64Ops &op, int &n,
-                                              bool n_small) {
-    const double2 c0 = ld_const2(tab + kConstExp), c1 = ld_const2(tab + kConstExp + 2),
-                  c2 = ld_const2(tab + kConstExp + 4), c3 = ld_const2(tab + kConstExp + 6);
-    const double t = fma(x, c0.x, c0.y);   // x * 256/ln2 + 1.5 * 2^52: rounded to an integer
-    n = (int)(unsigned)__double_as_longlong(t);
-    const double nd = n_small ? f2d_alu(small_int_to_float(n)) : op.sub(t, c0.y);
-    double r = fma(nd, c1.x, x);           // - n ln2/256, high 36 bits
-    r = fma(nd, c1.y, r);                  // low part
-    double p = fma(r, c2.x, c2.y);
-    p = fma(r, p, c3.x);
+// x = (256 k + j) ln2/256 + r with |r| about ln2/512, exp(x) = 2^k 2^(j/256)
+// e^r, 2^(j/256) from a 256-entry table and e^r - 1 = r (1 + r (1/2 + r t)).
+//   The FP64 pipe bounds the step, so only what needs 53 bits is left to it:
+// five operations.
+//   The integer n = 256 k + j is rounded in FP32 (near a half it may be the
+// next one, which only moves r past ln2/512, to 0.0014) and becomes a double
+// on the integer pipe.
+//   r is x less n times ln2/256 rounded to 53 bits: exact, a multiple of
+// 2^-61 below 2^-9.  What the constant lacks, d = -n 9.06e-20 of at most
+// 2e-14, is FP32's and comes as d (1 + r) with the last multiplication.
+//   t = 1/6 + r/24 is FP32 from r rounded, its error of 2^-27 standing behind
+// r^3 < 2^-28; its constant is two units above 1/6, which stands for the next
+// term's r^2/120.
+//   Against extended precision on [-64, 64] the largest error is 1.24 ulp and
+// the root mean square 0.418 ulp; with all of it in FP64 (eight operations, t
+// without the next term) they were 1.32 and 0.421.  exp_near: y 2^(n >> 8) =
+// exp(x) for |x| <= 1024.
+__device__ __forceinline__ double exp_near(double x, const double *tab, const Fp64Ops &op, int &n) {
+    const double2 c0 = ld_const2(tab + kConstExp);
+    const float z = fmaf(near_float(x), 369.32993f, 12582912.f);   // x * 256/ln2 + 1.5 * 2^23
+    n = __float_as_int(z) - 0x4b400000;
+    const float nf = z - 12582912.f;
+    const double r = fma(f2d_int(nf), c0.x, x);
+    const float rf = near_float(r), d = nf * -0x1.abc9e4p-64f;
+    double p = fma(r, f2d_pos(fmaf(rf, 0x1.555556p-5f, 0x1.555558p-3f)), c0.y);
     p = fma(r, p, op.one);
-    p = op.mul(p, r);                      // e^r - 1
+    p = fma(p, r, f2d_int(fmaf(d, rf, d)));   // e^r - 1
     const double s = __ldg(tab + (n & (kExpTab - 1)));
     return fma(s, p, s);
 }
@@ -227,28 +236,47 @@ __device__ __forceinline__ double fexp(double x, const double *tab, const Fp64Op
     const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32);
     if (((hi >> 20) & 0x7ffu) > 0x407u) return exp_outside(x);
     int n;
-    const double y = exp_reduced(x, tab, op, n, true);   // |n| < 2^18
+    const double y = exp_near(x, tab, op, n);   // |n| < 2^18
     const long long k = (long long)(n >> 8);
     return __longlong_as_double(__double_as_longlong(y) + (k << 52));
 }
 
 // exp(x) = y 2^k with y in [0.99, 2.01]: the reduction of fexp without its
 // final scaling, so that products of many exponentials can be formed
-// without overflow.  The reduction is exact up to its two roundings for
-// any |x| < 2^22 (the products with ln2/256 are fused, and the table index
-// fits an int); beyond that (and for infinities) k saturates at +-2^24 with
-// y = 1, and a NaN x gives a NaN y.
-__device__ __forceinline__ void split_exp(double x, const double *tab, const Fp64Ops &op, double &y, int &k) {
+// without overflow.  From |x| = 1024 on the reduction is in FP64 throughout:
+// exact up to its two roundings for any |x| < 2^22 (the products with
+// ln2/256 are fused, and the table index fits an int); beyond that (and for
+// infinities) k saturates at +-2^24 with y = 1, and a NaN x gives a NaN y.
+struct SplitExp {
+    double y;
+    int k;
+};
+static __device__ __noinline__ SplitExp split_exp_far(double x, const double *tab) {
     const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32);
     const unsigned ex = (hi >> 20) & 0x7ffu;
     if (ex >= 0x415u) {
         const bool nan = ex == 0x7ffu && ((hi & 0xfffffu) | (unsigned)__double_as_longlong(x));
-        y = nan ? x : 1.0;
-        k = (hi >> 31) ? -(1 << 24) : (1 << 24);
+        return SplitExp{nan ? x : 1.0, (hi >> 31) ? -(1 << 24) : (1 << 24)};
+    }
+    const double t = fma(x, 369.3299304675746, 6755399441055744.0);   // + 1.5 * 2^52: rounded to an integer
+    const int n = (int)(unsigned)__double_as_longlong(t);
+    const double nd = t - 6755399441055744.0;
+    double r = fma(nd, -0x1.62e42fefa0000p-9, x);   // ln2/256 in two parts
+    r = fma(nd, -0x1.cf79abc9e3b3ap-48, r);
+    const double p = r * fma(r, fma(r, fma(r, 1.0 / 24.0, 1.0 / 6.0), 0.5), 1.0);
+    const double s = __ldg(tab + (n & (kExpTab - 1)));
+    return SplitExp{fma(s, p, s), n >> 8};
+}
+__device__ __forceinline__ void split_exp(double x, const double *tab, const Fp64Ops &op, double &y, int &k) {
+    const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32);
+    if (((hi >> 20) & 0x7ffu) > 0x408u) {
+        const SplitExp f = split_exp_far(x, tab);
+        y = f.y;
+        k = f.k;
         return;
     }
     int n;
-    y = exp_reduced(x, tab, op, n, false);
+    y = exp_near(x, tab, op, n);
     k = n >> 8;
 }
 // v 2^k on the exponent bits for a normal v; zero, subnormal, infinite and
@@ -269,8 +297,10 @@ __device__ __forceinline__ double scale_pow2(double v, int k) {
 // 16(4), 1990: x = 2^k y with y in [1, 2), F = 1 + j/128 the table point
 // nearest to y (j = 0..128), f = y - F (exact, |f| <= 2^-8), u = f (1/F),
 // and ln x = k ln2 + ln F + ln(1 + u) with ln(1 + u) by its series to u^6
-// (truncation below 2^-56 / 7): ten FP64 operations, within 1.5 ulp.  {1/F,
-// ln F} come from a table; k becomes a double on the integer pipe.  (Below 2
+// (truncation below 2^-56 / 7), within 1.5 ulp.  The terms from u^4 on are
+// formed in FP32 (their error of 2^-26 stands behind u^4 < 2^-32, the result
+// is at least 0.69): eight FP64 operations.  {1/F, ln F} come from a table;
+// k becomes a double on the integer pipe.  (Below 2
 // the result can be small next to k ln2 + ln F, and the table's rounding
 // then leaves an absolute error near 1e-16.  The kernels take it of T in
 // [200, 6000] K.)
@@ -281,16 +311,14 @@ __device__ __forceinline__ double flog(double x, const double2 *tab, const doubl
     const int j = (int)((b >> 45) & 0x7f) + (int)((b >> 44) & 1);
     const double F = __longlong_as_double(0x3ff0000000000000LL + ((long long)j << 45));
     const double2 t = __ldg(tab + j);
-    const double2 c0 = ld_const2(exp_tab + kConstLog), c1 = ld_const2(exp_tab + kConstLog + 2),
-                  c2 = ld_const2(exp_tab + kConstLog + 4);
+    const double2 c1 = ld_const2(exp_tab + kConstLog), c2 = ld_const2(exp_tab + kConstLog + 2);
     const double u = op.mul(op.sub(y, F), t.x);
-    double p = fma(u, c0.x, c0.y);   // -1/6, 1/5
-    p = fma(u, p, c1.x);             // -1/4
-    p = fma(u, p, c1.y);             // 1/3
-    p = fma(u, p, c2.x);             // -1/2
+    const float uf = near_float(u), w = fmaf(uf, fmaf(uf, 1.f / 6.f, -0.2f), 0.25f);
+    double p = fma(-u, f2d_pos(w), c1.x);   // 1/3 - u (1/4 - u/5 + u^2/6)
+    p = fma(u, p, c1.y);                    // -1/2
     p = fma(u, p, op.one);
     const double kd = f2d_alu(small_int_to_float(k));
-    return fma(u, p, fma(kd, c2.y, t.y));   // ln 2
+    return fma(u, p, fma(kd, c2.x, t.y));   // ln 2
 }
 
 // NASA-7 entropy from the thermo coefficients of one species and range
