@@ -166,7 +166,7 @@ static void third_body_first(const chem_mech_desc *in, ReorderedMech &o) {
 struct HostTables {
     std::vector<double> thermo, tmid, tpoly, sp, rxn_d, eff_c, d_ce, j_c, exp_tab, log_tab;
     std::vector<unsigned> div16;
-    std::vector<float> tpoly_f;
+    std::vector<float> tpoly_f, cv_max;
     std::vector<float> rxn_df, d_cef, spf;
     std::vector<int2> d_pk, d_pk64;
     std::vector<unsigned> j_w, sp_w;
@@ -252,6 +252,29 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
             for (int i = 0; i <= 4; ++i) cf[i] = (float)c[6 + i];
             for (int i = 0; i <= 5; ++i) cf[5 + i] = (float)c[i];
         }
+    // the most by which a species' energy can change per kelvin of the
+    // temperature recovery's bracket: its largest c_v, sampled, a part in a
+    // thousand for what lies between the samples, and the step between the
+    // ranges over one kelvin
+    t.cv_max.resize(ns);
+    for (int s = 0; s < ns; ++s) {
+        auto poly = [&](int rg) { return &t.tpoly[((size_t)s * 2 + rg) * kTpolyStride]; };
+        double top = 0.0;
+        for (int Ti = (int)kTlo; Ti <= (int)kThi; Ti += 20)
+            for (int rg = 0; rg < 2; ++rg) {
+                if (rg == 0 ? Ti > d->t_mid[s] + 20 : Ti < d->t_mid[s] - 20) continue;
+                const double *c = poly(rg) + 6;
+                top = std::max(top, std::fabs((((c[4] * Ti + c[3]) * Ti + c[2]) * Ti + c[1]) * Ti + c[0]));
+            }
+        const double T = d->t_mid[s];
+        double step = 0.0;
+        if (T >= kTlo && T <= kThi)
+            for (int rg = 0; rg < 2; ++rg) {
+                const double *c = poly(rg);
+                step += (rg ? 1 : -1) * (((((c[5] * T + c[4]) * T + c[3]) * T + c[2]) * T + c[1]) * T + c[0]);
+            }
+        t.cv_max[s] = (float)(1.001 * top + std::fabs(step));
+    }
     // dense stoichiometry
     std::vector<int> nuR((size_t)nr * ns, 0), nuP((size_t)nr * ns, 0);
     for (int r = 0; r < nr; ++r)
@@ -639,7 +662,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
         return parts.size() - 1;
     };
     auto addv = [&](const auto &v) { return add(v.data(), v.size() * sizeof(v[0])); };
-    const size_t i_th = addv(t.thermo), i_tm = addv(t.tmid), i_tp = addv(t.tpoly), i_tpf = addv(t.tpoly_f),
+    const size_t i_th = addv(t.thermo), i_tm = addv(t.tmid), i_tp = addv(t.tpoly), i_tpf = addv(t.tpoly_f), i_cvm = addv(t.cv_max),
                  i_sp = addv(t.sp), i_rd = addv(t.rxn_d),
                  i_rf = addv(t.rxn_f), i_ep = addv(t.eff_ptr), i_es = addv(t.eff_sp), i_ec = addv(t.eff_c),
                  i_dpk = addv(t.d_pk),
@@ -689,6 +712,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
     m.tmid = (const double *)at(i_tm);
     m.tpoly = (const double *)at(i_tp);
     m.tpoly_f = (const float *)at(i_tpf);
+    m.cv_max = (const float *)at(i_cvm);
     m.sp = (const double *)at(i_sp);
     m.rxn_d = (const double *)at(i_rd);
     m.rxn_f = (const int *)at(i_rf);

@@ -133,6 +133,7 @@ struct DeviceMech {
     const double *thermo;       // [16][2][ns] (coefficient-major, above)
     const double *tmid;         // [ns] (positive: compared as integers)
     const double *tpoly;        // [12][2][ns] energy and heat-capacity polynomials
+    const float *cv_max;        // [ns] bound of c_v on [kTlo, kThi] (HostTables)
     const float *tpoly_f;       // [12][2][ns] heat-capacity and energy polynomials in FP32
     const double *sp;           // [ns][4]
     const double *rxn_d;        // [nr][4] ln A (SI), beta, E/R, sum nu

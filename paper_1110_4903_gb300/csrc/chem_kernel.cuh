@@ -324,7 +324,7 @@ __device__ __forceinline__ double flog(double x, const double2 *tab, const doubl
 // NASA-7 entropy from the thermo coefficients of one species and range
 // (layout in chem_internal.h)
 __device__ __forceinline__ double nasa_s(const CoefRow<double> &th, double T, double lnT, const Fp64Ops &op) {
-    return op.add(fma(th[0], lnT, op.mul(T, fma(T, fma(T, fma(T, th[12], th[11]), th[10]), th[1]))), th[13]);
+    return fma(th[0], lnT, fma(T, fma(T, fma(T, fma(T, th[12], th[11]), th[10]), th[1]), th[13]));
 }
 // Sums over a cell's species with one species per lane (wide warps, below),
 // in the order of G0 lanes per cell: lane l of those sums the terms l, l + G0,
@@ -370,6 +370,16 @@ __device__ __forceinline__ float wide_dotf(float a, float b, int cnt, float firs
 //   `cold` slots have no guess: where no density is negative (so that e(T) is
 // increasing and has one root) three Newton steps in FP32 find one, from
 // which two FP64 passes suffice instead of six.
+//   A diverging substep's densities, some negative and large, often have no
+// temperature, and halving the bracket down to one of its ends takes up to 48
+// passes to find that out: 36 species, mixed, 4 % of the recoveries took two
+// thirds of the passes.  So once a Newton step leaves the bracket, the
+// residual is held against the most that it can change over the bracket,
+// `slope` = sum |rho_s| max c_v,s (the energies' steps at t_mid included)
+// times its width: a larger one keeps its sign, and the passes would have
+// ended at the bracket's end, as this does.  (A hundredth of the width and of
+// a kelvin on top keep later Newton steps from ending inside the bracket
+// first: none could be below 0.01 K.)
 //   The energies come from the multiplied-out polynomials (five DFMA per
 //   species, no 1/T); with F32 the derivative sum c_v is formed in FP32, which
 //   changes the Newton steps by a relative 1e-7 and not the root.
@@ -382,6 +392,7 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
     if (!(bits_gt(T, lo) && bits_lt(T, hi))) T = 1500.0;
     bool done = !need;
     ok = false;
+    float slope = CUDART_INF_F;
     const double e = x[ns];
     if (__any_sync(kFull, cold)) {
         float Tf = 1500.f;
@@ -473,6 +484,7 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
                 fp = wide_dot<G0>(xs, fp, ns, op);
             rfp = frcp1(fp, op);
         }
+        bool left = false;
         if (!done) {
             const long long fb = __double_as_longlong(f);
             if ((fb << 1) == 0) {
@@ -492,6 +504,7 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
                 if (!inside && bits_gt(fabs(dT), tol)) {
                     Tn = 0.5 * (lo + hi);
                     dT = op.sub(Tn, T);
+                    left = true;
                 }
                 T = Tn;
                 if (!bits_gt(fabs(dT), tol)) {
@@ -499,6 +512,16 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
                     ok = bits_gt(T, kTlo * (1.0 + 1e-9)) && bits_lt(T, kThi * (1.0 - 1e-9));
                 }
             }
+        }
+        if (__any_sync(kFull, left)) {
+            if (__any_sync(kFull, left && slope == CUDART_INF_F)) {
+                slope = 0.f;
+#pragma unroll 1
+                for (int s = sl; s < ns; s += G) slope = fmaf(fabsf(d2f_rz(x[s])), __ldg(m.cv_max + s), slope);
+                slope = Grp<G>::sum(slope);
+            }
+            // (infinities and NaN compare false)
+            if (left && fabsf(d2f_rz(f)) > slope * fmaf(1.01f, d2f_rz(hi) - d2f_rz(lo), 0.01f)) done = true;
         }
     }
     if (need) T_out = T;
