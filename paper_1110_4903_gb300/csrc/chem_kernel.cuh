@@ -1885,44 +1885,48 @@ __device__ __forceinline__ void step_cells(const DeviceMech &m, const StepOption
             }
             int act = state == kRejected ? kFailSubstep : kNoAction, code = kCellOk;
             bool advanced = false;   // the cell reached dt: its state is written
-            int nonfin = 0;
-            double rt = 0.0, es = 0.0;
-            if (loading) {
-                iters = subs = fails = 0;
-                Tin = CUDART_NAN;
-                if (!Q && b.schedule && sl == 0) {
+            // (with no cell to load, the sums' FP64 additions would be a twentieth of
+            // all of an iteration's)
+            if (__any_sync(kFull, loading)) {
+                int nonfin = 0;
+                double rt = 0.0, es = 0.0;
+                if (loading) {
+                    iters = subs = fails = 0;
+                    Tin = CUDART_NAN;
+                    if (!Q && b.schedule && sl == 0) {
 #pragma unroll 1
-                    for (int w = 0; w < kSchedWords; ++w) b.schedule[cell * kSchedWords + w] = 0u;
-                }
+                        for (int w = 0; w < kSchedWords; ++w) b.schedule[cell * kSchedWords + w] = 0u;
+                    }
 #pragma unroll 1
-                for (int i = sl; i < n; i += G) {
-                    const double v = i < ns ? rho_in[(size_t)i * ld_in + cell] : e_in[cell];
-                    sm.x0[i] = v;
-                    sm.x[i] = v;
-                    if (!isfinite(v)) nonfin = 1;
-                    const double ev = fabs(i < ns ? v * __ldg(m.sp + i * kSpStride + 3) : v);
-                    if (i < ns) rt = G == G0 ? rt + v : v;
-                    es = G == G0 ? es + ev : ev;
+                    for (int i = sl; i < n; i += G) {
+                        const double v = i < ns ? rho_in[(size_t)i * ld_in + cell] : e_in[cell];
+                        sm.x0[i] = v;
+                        sm.x[i] = v;
+                        if (!isfinite(v)) nonfin = 1;
+                        const double ev = fabs(i < ns ? v * __ldg(m.sp + i * kSpStride + 3) : v);
+                        if (i < ns) rt = G == G0 ? rt + v : v;
+                        es = G == G0 ? es + ev : ev;
+                    }
                 }
-            }
-            nonfin = Grp<G>::any(nonfin);
-            if constexpr (G == G0) {
-                rt = Grp<G>::sum(rt);
-                es = Grp<G>::sum(es);
-            } else {
-                const Fp64Ops op = fp64_ops(tab);
-                rt = wide_dot<G0>(rt, op.one, ns, op);
-                es = wide_dot<G0>(es, op.one, n, op);
-            }
-            if (loading) {
-                atol_rho = o.atol_rel * rt;
-                atol_e = o.atol_rel * es;
-                T = (!Q && b.T_in) ? b.T_in[cell] : 1500.0;
-                if (nonfin || !(rt > 0.0)) {
-                    act = kEmitCell;
-                    code = kCellBadInput;
+                nonfin = Grp<G>::any(nonfin);
+                if constexpr (G == G0) {
+                    rt = Grp<G>::sum(rt);
+                    es = Grp<G>::sum(es);
                 } else {
-                    state = kInitT;
+                    const Fp64Ops op = fp64_ops(tab);
+                    rt = wide_dot<G0>(rt, op.one, ns, op);
+                    es = wide_dot<G0>(es, op.one, n, op);
+                }
+                if (loading) {
+                    atol_rho = o.atol_rel * rt;
+                    atol_e = o.atol_rel * es;
+                    T = (!Q && b.T_in) ? b.T_in[cell] : 1500.0;
+                    if (nonfin || !(rt > 0.0)) {
+                        act = kEmitCell;
+                        code = kCellBadInput;
+                    } else {
+                        state = kInitT;
+                    }
                 }
             }
             __syncwarp();
