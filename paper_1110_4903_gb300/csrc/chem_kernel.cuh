@@ -324,7 +324,7 @@ __device__ __forceinline__ double flog(double x, const double2 *tab, const doubl
 // NASA-7 entropy from the thermo coefficients of one species and range
 // (layout in chem_internal.h)
 __device__ __forceinline__ double nasa_s(const CoefRow<double> &th, double T, double lnT, const Fp64Ops &op) {
-    return fma(th[0], lnT, fma(T, fma(T, fma(T, fma(T, th[12], th[11]), th[10]), th[1]), th[13]));
+    return op.add(fma(th[0], lnT, op.mul(T, fma(T, fma(T, fma(T, th[12], th[11]), th[10]), th[1]))), th[13]);
 }
 // Sums over a cell's species with one species per lane (wide warps, below),
 // in the order of G0 lanes per cell: lane l of those sums the terms l, l + G0,
