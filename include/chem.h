@@ -417,6 +417,10 @@ int chem_selftest_log(int64_t n, const double *x, double *y_log, double *y_log_r
 int chem_selftest_scaled_exp(int64_t n, const double *x, double *y_mant, int32_t *y_pow,
                              const double *v, const int32_t *k, double *y_scaled, void *stream);
 
+/* Diagnostics: the step kernel's sum over a warp, y[i] the sum of the 32
+ * device values x[32 i], ..., x[32 i + 31].  Synchronous. */
+int chem_selftest_warp_sum(int64_t n, const double *x, double *y, void *stream);
+
 /* Human-readable text for a CHEM_E_* code (static storage). */
 const char *chem_strerror(int code);
 

@@ -126,6 +126,7 @@ def lib():
             "chem_batched_solve": [i32, i32, i64, p, p, p, p, p],
             "chem_selftest_math": [i64, p, p, p, p, p, p],
             "chem_selftest_log": [i64, p, p, p, p],
+            "chem_selftest_warp_sum": [i64, p, p, p],
             "chem_selftest_scaled_exp": [i64, p, p, p, p, p, p, p],
         }
         for name, args in sig.items():

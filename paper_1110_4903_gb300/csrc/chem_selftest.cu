@@ -1,6 +1,6 @@
 // chem_selftest.cu -- diagnostics: the step kernel's own exp, logarithm and
-// reciprocal evaluated next to CUDA's, and its split exponential and
-// power-of-two scaling, so tests can bound their error and check their range
+// reciprocal evaluated next to CUDA's, its split exponential and power-of-two
+// scaling, and its sum over a warp, so tests can bound their error and check their range
 // handling.
 #include <cuda_runtime.h>
 
@@ -46,6 +46,14 @@ __global__ void selftest_log_kernel(long long n, const double *x, const double2 
     y_log_ref[i] = log(x[i]);
 }
 
+__global__ void selftest_warp_sum_kernel(long long n, const double *x, const double *tab, double *y) {
+    const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    if (row >= n) return;
+    const int lane = threadIdx.x & 31;
+    const double s = Grp<32>::sum<true>(x[row * 32 + lane], fp64_ops(tab));
+    if (lane == 0) y[row] = s;
+}
+
 }  // namespace chem
 
 using namespace chem;
@@ -85,6 +93,20 @@ extern "C" int chem_selftest_log(int64_t n, const double *x, double *y_log, doub
     }
     cudaFree(d_tab);
     cudaFree(d_exp);
+    if (ce != cudaSuccess) return cuda_fail(ce, "self-test");
+    return CHEM_OK;
+}
+
+extern "C" int chem_selftest_warp_sum(int64_t n, const double *x, double *y, void *stream) {
+    if (n < 0 || !x || !y) return fail(CHEM_E_INVALID_ARG, "NULL argument");
+    if (n == 0) return CHEM_OK;
+    double *d_tab = nullptr;
+    const int rc = upload_exp_table(&d_tab);
+    if (rc) return rc;
+    selftest_warp_sum_kernel<<<(unsigned)((n + 7) / 8), 256, 0, (cudaStream_t)stream>>>(n, x, d_tab, y);
+    cudaError_t ce = cudaGetLastError();
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize((cudaStream_t)stream);
+    cudaFree(d_tab);
     if (ce != cudaSuccess) return cuda_fail(ce, "self-test");
     return CHEM_OK;
 }
