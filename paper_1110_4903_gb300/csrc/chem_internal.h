@@ -92,9 +92,10 @@ constexpr int kLogTab = 128;
 //           once per Jacobian entry in the gather
 // Gather lists laid out for G lanes per cell.  List p (a Jacobian entry, or
 // an item of a species list) runs in pass p / G on lane p % G; its q-th term
-// sits at word base + q G + lane, where base is the pass's first word, so the
-// lanes of a pass read their q-th terms from consecutive words (one cache
-// line per warp load instead of one per lane).
+// sits at word base + 4 ((q / 4) G + lane) + q % 4, where base is the pass's
+// first word, so the lanes of a pass read four terms each from consecutive
+// words with one 16-byte load.  Zeros fill a list's place up to the whole
+// chunks of its pass's longest.
 //   The ns*ns species entries (the kernels eliminate the energy unknown, so
 //   no energy row is gathered), longest list first, in both forms:
 //     j_meta[p]   = {first word of entry p, k | s << 8 | terms << 16}

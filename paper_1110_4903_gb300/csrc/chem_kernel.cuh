@@ -1035,7 +1035,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         sm.Q[r] = f32 || tb ? op.mul(CM, q) : q;   // in the D region until phase 4
         if (f32) {
             // Jacobian-only quantities in FP32 from FP32 copies
-            const float *rf = m.rxn_df + (size_t)r * kRxnDStride;
+            const float4 rf = __ldg(reinterpret_cast<const float4 *>(m.rxn_df) + r);
             // (products formed in FP32 from converted factors: the FP64
             // pipe keeps to the rates the residual needs)
             const JT CMf = to_jt<JT>(CM);
@@ -1045,8 +1045,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             if (r < m.ntb) sm.qtb[r] = to_jt<JT>(q);
             const JT shf = s3 ? (sm.hJ[b0] + sm.hJ[b1] + sm.hJ[b2]) - (sm.hJ[a0] + sm.hJ[a1] + sm.hJ[a2])
                               : (sm.hJ[b0] + sm.hJ[b1]) - (sm.hJ[a0] + sm.hJ[a1]);
-            const JT dlnkf = (JT)__ldg(rf + 1) * iT * iT + (JT)__ldg(rf) * iT;
-            const JT dlnKc = (shf - (JT)__ldg(rf + 2)) * iT;
+            const JT dlnkf = fmaf(rf.y * iT, iT, __fmul_rn(rf.x, iT));
+            const JT dlnKc = (shf - (JT)rf.z) * iT;
             // concentration products again in FP32 (a conversion costs an
             // FP64-pipe slot, three FP32 products do not)
             JT PfJ = sm.cJ[a0] * sm.cJ[a1], PbJ = sm.cJ[b0] * sm.cJ[b1];
@@ -1080,18 +1080,12 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
     const GatherLayout &gl = m.gl[layout_index(G)];
     const unsigned *gl_j_w = G == G0 ? gl.j_w : m.j_w_wide[layout_index(G0)];
     //   The table's words come from L2 as often as from L1, so an item's
-    //   eight words are loaded together, the next item's descriptor with
-    //   them, and the operands of four terms at a time; the sums keep the
-    //   order of the list.
+    //   words are loaded four at a time (16 bytes), the next item's
+    //   descriptor with them, and the operands of four terms at a time; the
+    //   sums keep the order of the list.
     auto item_at = [&](int it) -> int2 { return it < m.n_items ? __ldg(gl.it_meta + it) : make_int2(0, 0); };
     auto item_words = [&](int e, int rem) -> uint4 {
-        const unsigned *wp = gl.sp_w + e;
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (rem > 0) w.x = __ldg(wp);
-        if (rem > 1) w.y = __ldg(wp + G);
-        if (rem > 2) w.z = __ldg(wp + 2 * G);
-        if (rem > 3) w.w = __ldg(wp + 3 * G);
-        return w;
+        return rem > 0 ? __ldg(reinterpret_cast<const uint4 *>(gl.sp_w + e)) : make_uint4(0u, 0u, 0u, 0u);
     };
     static_assert(kChunk == 8, "an item is two groups of four terms");
     int2 im = item_at(sl);
@@ -1333,8 +1327,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         const int nnz = m.nJ_nz;
         auto meta_at = [&](int p) -> int4 { return p < nnz ? __ldg(gl.j_meta32 + p) : make_int4(0, 0, 0, 0); };
         auto words_at = [&](int e) -> uint4 {
-            const unsigned *wp = gl_j_w + e;
-            return make_uint4(__ldg(wp), __ldg(wp + G), __ldg(wp + 2 * G), __ldg(wp + 3 * G));
+            return __ldg(reinterpret_cast<const uint4 *>(gl_j_w + e));
         };
         int4 me = meta_at(sl), mn = meta_at(sl + G);
         uint4 wn = words_at(me.x);
@@ -1349,8 +1342,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             float a0 = 0.f, a1 = 0.f;
 #pragma unroll 1
             do {
-                const unsigned x0 = rem > 0 ? w.x : 0u, x1 = rem > 1 ? w.y : 0u, x2 = rem > 2 ? w.z : 0u,
-                               x3 = rem > 3 ? w.w : 0u;
+                const unsigned x0 = w.x, x1 = w.y, x2 = w.z, x3 = w.w;
                 const bool whole = rem > 3;
                 const float v0 = Dv[x0 & 0x7fffffu], v1 = Dv[x1 & 0x7fffffu], v2 = Dv[x2 & 0x7fffffu],
                             v3 = Dv[x3 & 0x7fffffu];
@@ -1372,15 +1364,15 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         // -h, the initial values the identity and u: two FP64 operations per
         // entry beside its terms)
         struct Terms {
-            int d[4];
-            double c[4];
+            int4 d;
+            double2 c0, c1;
         };
         auto terms_at = [&](int e, int rem) -> Terms {
-            Terms t;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                t.d[i] = rem > i ? __ldg(gl.j_d + e + i * G) : 0;
-                t.c[i] = rem > i ? __ldg(gl.j_c + e + i * G) : 0.0;
+            Terms t{make_int4(0, 0, 0, 0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+            if (rem > 0) {
+                t.d = __ldg(reinterpret_cast<const int4 *>(gl.j_d + e));
+                t.c0 = __ldg(reinterpret_cast<const double2 *>(gl.j_c + e));
+                t.c1 = __ldg(reinterpret_cast<const double2 *>(gl.j_c + e) + 1);
             }
             return t;
         };
@@ -1403,16 +1395,16 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             if (len > 0) {
 #pragma unroll 1
                 for (;;) {
-                    const double v0 = Dv[t.d[0]], v1 = Dv[t.d[1]], v2 = Dv[t.d[2]], v3 = Dv[t.d[3]];
+                    const double v0 = Dv[t.d.x], v1 = Dv[t.d.y], v2 = Dv[t.d.z], v3 = Dv[t.d.w];
                     const Terms tc = t;
                     const int rc = rem;
                     rem -= 4;
                     e += 4 * G;
                     t = terms_at(e, rem);
-                    ua = fma(tc.c[0], v0, ua);
-                    if (rc > 1) ua = fma(tc.c[1], v1, ua);
-                    if (rc > 2) ua = fma(tc.c[2], v2, ua);
-                    if (rc > 3) ua = fma(tc.c[3], v3, ua);
+                    ua = fma(tc.c0.x, v0, ua);
+                    if (rc > 1) ua = fma(tc.c0.y, v1, ua);
+                    if (rc > 2) ua = fma(tc.c1.x, v2, ua);
+                    if (rc > 3) ua = fma(tc.c1.y, v3, ua);
                     if (rem <= 0) break;
                 }
             }
