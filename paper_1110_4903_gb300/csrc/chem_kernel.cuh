@@ -999,12 +999,7 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         const bool s3 = __any_sync(__activemask(), (a2 != ns) | (b2 != ns));
         double Pf = op.mul(sm.c[a0], sm.c[a1]);
         double Pb = op.mul(sm.c[b0], sm.c[b1]);
-        // (the FP64 path rounds E/RT and the forward rate by themselves: its
-        // temperature derivatives use them too)
-        const double EaRT = f32 ? 0.0 : op.mul(EaR, invT);
-        const double lnAT = fma(beta, lnT, lnA);
-        const double lnkf = f32 ? fma(-EaR, invT, lnAT) : op.sub(lnAT, EaRT);
-        const double kf = fexp(lnkf, tab, op);
+        const double kf = fexp(fma(-EaR, invT, fma(beta, lnT, lnA)), tab, op);
         // K_b = K_f / K_c with 1/K_c = (RT/P_a)^dnu exp(dG/RT) (Eq. 24) as
         // the product over the factor slots of the species' exp(g/RT) (RT/P_a)
         // (products) and their inverses (reactants), the sentinel giving 1:
@@ -1030,8 +1025,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
 #pragma unroll 1
             for (int e = e0; e < e1; ++e) CM = fma(__ldg(m.eff_c + e), sm.c[__ldg(m.eff_sp + e)], CM);
         }
-        const double rev = op.mul(kb, Pb), fwd = f32 ? 0.0 : op.mul(kf, Pf);
-        const double q = f32 ? fma(kf, Pf, -rev) : op.sub(fwd, rev);
+        const double rev = op.mul(kb, Pb);
+        const double q = fma(kf, Pf, -rev);
         sm.Q[r] = f32 || tb ? op.mul(CM, q) : q;   // in the D region until phase 4
         if (f32) {
             // Jacobian-only quantities in FP32 from FP32 copies
@@ -1060,15 +1055,16 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             // nothing: -h C_M k_f, -h C_M k_b, -h q_tb, and -h T dQ/dT (the
             // species' sums take the 1/T)
             //   T dln k_f/dT = beta + E/RT,
-            //   T dln k_b/dT = that less sum nu (h/RT - 1)
+            //   T dln k_b/dT = that less sum nu (h/RT - 1),
+            // so that T dQ/dT = C_M (q (beta + E/RT) + reverse rate times the
+            // sum): three operations fewer than from both rates
             const double hb = op.add(sm.hRT[b0], sm.hRT[b1]), ha = op.add(sm.hRT[a0], sm.hRT[a1]);
             const double sh = s3 ? op.sub(op.add(hb, sm.hRT[b2]), op.add(ha, sm.hRT[a2])) : op.sub(hb, ha);
             const double CMh = tb ? op.mul(CM, -h) : -h;
             if (r < m.ntb) sm.qtb[r] = (JT)op.mul(q, -h);
             sm.A1[r] = (JT)op.mul(CMh, kf);
             sm.A2[r] = (JT)op.mul(CMh, kb);
-            const double dlf = op.add(beta, EaRT);
-            sm.dQdT[r] = (JT)op.mul(CMh, fma(fwd, dlf, -op.mul(rev, op.sub(dlf, sh))));
+            sm.dQdT[r] = (JT)op.mul(CMh, fma(q, fma(EaR, invT, beta), op.mul(rev, sh)));
         }
     }
     __syncwarp();
