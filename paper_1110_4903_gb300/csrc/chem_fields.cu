@@ -31,7 +31,8 @@ __device__ __forceinline__ void stage_tpoly(const DeviceMech &m, double *tab) {
     }
 }
 
-// 524,365 cells of 36 species: 1.75 ms with h/RT and two reads of Y, 0.35 ms so.
+// Bound by the FP64 pipe (five operations per species) and by memory alike.
+// 524,365 cells of 36 species: 0.43 ms with h/RT and two reads of Y, 0.29 ms so.
 __global__ void __launch_bounds__(kFieldThreads) state_from_tpy_kernel(DeviceMech m, long long n, long long ld,
                                                                        const double *T, const double *P,
                                                                        const double *Y, double *rho, double *e) {
@@ -72,9 +73,13 @@ __global__ void __launch_bounds__(kFieldThreads) state_from_tpy_kernel(DeviceMec
 // bisection on [kTlo, kThi], ended as in the step.  Without
 // a guess, and where no density is negative (so that e(T) is increasing and
 // has one root), Newton runs in FP32 first, at a sixty-fourth of the cost: from
-// 1500 K the FP64 iterations were six or seven, from there they are three.
-// 524,365 cells of 36 species: 5.0 ms with c_p/R and h/RT re-read from L2,
-// 1.1 ms so.
+// 1500 K the FP64 iterations were six or seven, from there they are two.
+// Bound by the FP64 pipe: after a step below a millionth of T the derivative
+// is kept (it has changed by as much, and the next step is below 1e-12 T), so
+// that the last iteration evaluates the energies alone.
+// 524,365 cells of 36 species: 6.4 ms with c_p/R and h/RT re-read from L2 and
+// the FP64 iterations from 1500 K, 0.81 ms without, 0.70 ms with one
+// derivative.
 __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m, long long n, long long ld,
                                                                     const double *rho, const double *e,
                                                                     const double *Tg, double *Tout) {
@@ -123,19 +128,32 @@ __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m
         const double Ts = f2d_alu(Tf);
         if (Ts > lo && Ts < hi) T = Ts;
     }
-    bool ok = false;
+    bool ok = false, near = false;
+    double slope = 0.0;   // 1 / (df/dT)
 #pragma unroll 1
     for (int it = 1; it <= kTmaxIter; ++it) {
         const long long Tb = __double_as_longlong(T);
-        double f = 0.0, fp = 0.0;
+        double f = 0.0;
+        if (near) {
 #pragma unroll 2
-        for (int s = 0; s < ns; ++s) {
-            const double2 *c =
-                reinterpret_cast<const double2 *>(tab + (2 * s + thermo_range(m, s, Tb)) * kEnergyCoefs);
-            const double2 c01 = c[0], c23 = c[1], c45 = c[2], d01 = c[3], d23 = c[4], d4 = c[5];
-            const double r = x[s * bs];
-            f = fma(r, fma(fma(fma(fma(fma(c45.y, T, c45.x), T, c23.y), T, c23.x), T, c01.y), T, c01.x), f);
-            fp = fma(r, fma(fma(fma(fma(d4.x, T, d23.y), T, d23.x), T, d01.y), T, d01.x), fp);
+            for (int s = 0; s < ns; ++s) {
+                const double2 *c =
+                    reinterpret_cast<const double2 *>(tab + (2 * s + thermo_range(m, s, Tb)) * kEnergyCoefs);
+                const double2 c01 = c[0], c23 = c[1], c45 = c[2];
+                f = fma(x[s * bs], fma(fma(fma(fma(fma(c45.y, T, c45.x), T, c23.y), T, c23.x), T, c01.y), T, c01.x), f);
+            }
+        } else {
+            double fp = 0.0;
+#pragma unroll 2
+            for (int s = 0; s < ns; ++s) {
+                const double2 *c =
+                    reinterpret_cast<const double2 *>(tab + (2 * s + thermo_range(m, s, Tb)) * kEnergyCoefs);
+                const double2 c01 = c[0], c23 = c[1], c45 = c[2], d01 = c[3], d23 = c[4], d4 = c[5];
+                const double r = x[s * bs];
+                f = fma(r, fma(fma(fma(fma(fma(c45.y, T, c45.x), T, c23.y), T, c23.x), T, c01.y), T, c01.x), f);
+                fp = fma(r, fma(fma(fma(fma(d4.x, T, d23.y), T, d23.x), T, d01.y), T, d01.x), fp);
+            }
+            slope = 1.0 / fp;
         }
         f = op.sub(f, ei);
         if (f == 0.0) {
@@ -146,7 +164,7 @@ __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m
             hi = T;
         else
             lo = T;
-        double Tn = T - f / fp, dT = Tn - T;
+        double Tn = fma(-f, slope, T), dT = Tn - T;
         const bool inside = Tn > lo && Tn < hi;
         const double tol = (inside ? kTstep : kTtol) * T;
         // (a step below half an ulp leaves T at an end of the bracket)
@@ -154,6 +172,7 @@ __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m
             Tn = 0.5 * (lo + hi);
             dT = Tn - T;
         }
+        near = inside && fabs(dT) <= 1e-6 * T;
         T = Tn;
         if (fabs(dT) <= tol) {
             ok = !(T <= kTlo * (1.0 + 1e-9) || T >= kThi * (1.0 - 1e-9));

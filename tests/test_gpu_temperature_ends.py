@@ -67,3 +67,26 @@ def test_recovery_beyond_the_bracket(torch, name, mixed):
     assert (st[up] == chem.CELL_OK).all()
     for c in np.nonzero(up)[0]:
         assert abs(og["T"][400 + c] - np.interp(0.0, r[c], T)) < 1e-2
+
+
+@pytest.mark.parametrize("name", ["h2air-1M", "hc36-256k"])
+def test_field_temperature_from_near_and_far_guesses(torch, name):
+    """A guess off by nothing, a rounding, up to the whole bracket, or none:
+    the same temperature (1e-12: the energy's rounding over its slope)."""
+    import parity as P
+    from paper_1110_4903_gb300 import chem, synth
+    mech, field, dt = synth.workload(name)
+    f = synth.subsample(field, np.arange(1003))
+    f.T[:8] = [200.001, 200.1, 999.999, 1000.0, 1000.001, 3000.0, 5999.9, 5999.999]
+    rho, e = P.initial_state(mech, f)
+    ch = chem.Chem(mech)
+    dev = torch.device("cuda")
+    r, ev = torch.tensor(rho, device=dev), torch.tensor(e, device=dev)
+    off = np.array([0.0, 1e-16, 1e-12, 1e-9, 3e-8, 0.9e-6, 1.1e-6, 1e-4, 1e-2, 0.5, -1e-6, -1e-3, -0.7])
+    guess = np.clip(f.T * (1.0 + off[np.arange(1003) % off.size]), 150.0, 7000.0)
+    for g in (None, guess):
+        out = torch.zeros(1003, dtype=torch.float64, device=dev)
+        ch.temperature(r, ev, out, **({} if g is None else {"T_guess": torch.tensor(g, device=dev)}))
+        torch.cuda.synchronize()
+        assert np.abs(out.cpu().numpy() / f.T - 1.0).max() < 1e-12
+    ch.close()
