@@ -395,7 +395,7 @@ int chem_batched_solve(int32_t method, int32_t n, int64_t n_sys, double *A, doub
                        int32_t *pivots, int32_t *info, void *stream);
 
 /* Diagnostics: evaluates the step kernel's own exp (table-driven, after
- * Tang) and reciprocal (rcp.approx + two Newton steps) at n device points x,
+ * Tang) and reciprocal (rcp.approx + one cubic correction) at n device points x,
  * next to CUDA's exp and IEEE division, for tests of their error.
  * Synchronous. */
 int chem_selftest_math(int64_t n, const double *x, double *y_exp, double *y_exp_ref,

@@ -508,11 +508,15 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
     for (size_t e = 0; e < t.j_d32.size(); ++e) t.j_w.push_back(fword(t.j_d32[e], t.j_nu[e]));
     for (size_t e = 0; e < t.sp_r.size(); ++e) t.sp_w.push_back(dword(t.sp_r[e], t.sp_nui[e]));
     // the gather layouts for each lane count (chem_internal.h): list p on
-    // lane p % G of pass p / G; the pass's terms lie in chunks of four per
-    // lane, lane after lane, so that a lane reads a chunk with 16 bytes (the
-    // term q at base + 4 ((q / 4) G + lane) + q % 4), zeros where a list ends.
-    // One load instead of four, 2^20 cells of 9 species (mixed): 21.2 -> 20.9
-    // ms, 152 of 36 species 4.44 -> 4.39 ms, 16,384 FP64 90.7 -> 90.3 ms.
+    // lane p % G of pass p / G; the pass's terms lie in chunks of `per` words
+    // per lane, lane after lane (the term q at base + per ((q / per) G + lane)
+    // + q % per), zeros where a list ends.  The species lists and the FP64
+    // lists have per = 4, so that a lane reads a chunk with 16 bytes: 2^20
+    // cells of 9 species (mixed) 21.2 -> 20.9 ms, 152 of 36 species 4.44 ->
+    // 4.39 ms, 16,384 FP64 90.7 -> 90.3 ms.  The FP32 lists have per = 1: they
+    // are short (3.6 terms on average), and their padding to fours costs more
+    // in L1 misses than the loads saved (65,536 cells of 36 species: 93.8
+    // against 92.8 ms).
     //   With `bank` (the shared-memory bank each term's operand sits in), the
     // terms of each list are put in an order in which the lanes of a pass
     // read distinct banks at each step where they can: the sum is the same
@@ -522,7 +526,7 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
     auto interleave = [](int nlists, const std::vector<int> &ptr, int G, std::vector<int2> &meta,
                          std::vector<int> &pos, int tag_shift, const std::vector<int> *tags,
                          const std::vector<int> *bank = nullptr, std::vector<int> *rank = nullptr,
-                         const std::vector<int> *given = nullptr) {
+                         const std::vector<int> *given = nullptr, int per = 4) {
         if (rank) rank->assign(ptr.back(), 0);
         int base = 0;
         pos.assign(ptr.back(), -1);
@@ -576,13 +580,13 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
                 for (int e = ptr[P0]; e < ptr[P1]; ++e) (*rank)[e] = slot[e - ptr[P0]];
             for (int q = P0; q < P1; ++q) {
                 const int len = ptr[q + 1] - ptr[q], lane = q - P0;
-                meta.push_back(make_int2(base + 4 * lane, (tags ? (*tags)[q] : 0) | (len << tag_shift)));
+                meta.push_back(make_int2(base + per * lane, (tags ? (*tags)[q] : 0) | (len << tag_shift)));
                 for (int e = ptr[q]; e < ptr[q + 1]; ++e) {
                     const int i = slot[e - ptr[P0]];
-                    pos[e] = base + 4 * ((i >> 2) * G + lane) + (i & 3);
+                    pos[e] = base + per * ((i / per) * G + lane) + i % per;
                 }
             }
-            base += ((maxlen + 3) & ~3) * G;
+            base += (maxlen + per - 1) / per * per * G;
         }
         return base;
     };
@@ -599,7 +603,7 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
         }
         std::vector<int2> meta32;
         std::vector<int> rank;
-        const int nw32 = interleave(ns * ns, t.j_ptr32, G, meta32, pos, 16, &t.j_sk32, &t.j_d32, &rank);
+        const int nw32 = interleave(ns * ns, t.j_ptr32, G, meta32, pos, 16, &t.j_sk32, &t.j_d32, &rank, nullptr, 1);
         // the FP32 entries' metadata: first word, length, offset of (s, k)
         // in the column-major matrix of columns of ldc rows, and the factor
         // M_s / M_k rounded once to FP32
@@ -617,7 +621,7 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
         if (ns < 32) {
             // the same order of terms for wide warps
             std::vector<int2> meta_w;
-            const int nww = interleave(ns * ns, t.j_ptr32, 32, meta_w, pos, 16, &t.j_sk32, nullptr, nullptr, &rank);
+            const int nww = interleave(ns * ns, t.j_ptr32, 32, meta_w, pos, 16, &t.j_sk32, nullptr, nullptr, &rank, 1);
             L.j_w_wide.assign(nww + 8 * 32, 0u);
             for (size_t e = 0; e < pos.size(); ++e) L.j_w_wide[pos[e]] = t.j_w[e];
         } else {

@@ -63,7 +63,7 @@ constexpr int kRxnFStride = 2;
 constexpr int kChunk = 8;
 
 // Threads per block of the step kernel at most (its launch bounds: two
-// such blocks per SM, at most 102 registers per thread).
+// such blocks per SM, at most 96 registers per thread).
 constexpr int kMaxBlockThreads = 320;
 
 // Entries of the exp table (2^(j/kExpTab)).
@@ -95,7 +95,8 @@ constexpr int kLogTab = 128;
 // sits at word base + 4 ((q / 4) G + lane) + q % 4, where base is the pass's
 // first word, so the lanes of a pass read four terms each from consecutive
 // words with one 16-byte load.  Zeros fill a list's place up to the whole
-// chunks of its pass's longest.
+// chunks of its pass's longest.  (The FP32 Jacobian lists: at base + q G +
+// lane, one word per load.)
 //   The ns*ns species entries (the kernels eliminate the energy unknown, so
 //   no energy row is gathered), longest list first, in both forms:
 //     j_meta[p]   = {first word of entry p, k | s << 8 | terms << 16}

@@ -26,9 +26,12 @@
 // path (JT = float) keeps the FP64 residual, rates, sources and
 // temperature, and moves everything that only feeds the Jacobian to FP32;
 // it writes the Jacobian's rank-two part and the identity densely, four
-// rows per store, then adds the sparse reaction sums, and its LU is
-// organised by columns.  It is bound by latency, so its slot layout is cut
-// to what it reads (20 warps per SM at 36 species).
+// rows per store, then adds the sparse reaction sums, and its LU is in
+// registers (24 to 36 unknowns) or organised by columns.  It is bound by
+// latency and by the FP64 pipe (57 % busy), so its slot layout is cut to what
+// it reads (20 warps per SM at 36 species), and its FP32 arithmetic keeps its
+// order to the bit: another rounding of the Jacobian changes the substep
+// schedules of some 4 % of the cells.
 //   Code size: with 20 warps at different phases, the instructions of one
 // Newton iteration have to stay in the SM's instruction caches.  The
 // compiler's unrolling of the many short runtime-count loops made the mixed
@@ -623,8 +626,10 @@ __device__ __forceinline__ void lu_update_colmajor(float *A, int ld, int n, int 
 // pivots and roundings of lu_update_colmajor.  The results move one register
 // down, so that column j is always in register 0 and the loop body is one
 // copy of the code.  The solution goes to A[N ld ...].
-//   Bound by latency.  A branch costs a warp some thirty cycles here, so the
-// body is straight-line: registers past the live columns are carried along
+//   Bound by latency: 36 unknowns take 25,900 cycles with one warp on the SM
+// and 41,600 with 20, in shared memory 43,800 and 57,500 before back
+// substitution.  A branch costs a warp some thirty cycles here, so the body is
+// straight-line: registers past the live columns are carried along
 // (what they hold is never used), rows of U may run past their end into the
 // next row's place, and only whole groups of eight columns are skipped.
 constexpr int kLuRegMinN = 24, kLuRegN = 36;
@@ -1323,7 +1328,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
         const int nnz = m.nJ_nz;
         auto meta_at = [&](int p) -> int4 { return p < nnz ? __ldg(gl.j_meta32 + p) : make_int4(0, 0, 0, 0); };
         auto words_at = [&](int e) -> uint4 {
-            return __ldg(reinterpret_cast<const uint4 *>(gl_j_w + e));
+            const unsigned *wp = gl_j_w + e;
+            return make_uint4(__ldg(wp), __ldg(wp + G), __ldg(wp + 2 * G), __ldg(wp + 3 * G));
         };
         int4 me = meta_at(sl), mn = meta_at(sl + G);
         uint4 wn = words_at(me.x);
@@ -1338,7 +1344,8 @@ __device__ void newton_iteration(const DeviceMech &m, const double *tab, SlotMem
             float a0 = 0.f, a1 = 0.f;
 #pragma unroll 1
             do {
-                const unsigned x0 = w.x, x1 = w.y, x2 = w.z, x3 = w.w;
+                const unsigned x0 = rem > 0 ? w.x : 0u, x1 = rem > 1 ? w.y : 0u, x2 = rem > 2 ? w.z : 0u,
+                               x3 = rem > 3 ? w.w : 0u;
                 const bool whole = rem > 3;
                 const float v0 = Dv[x0 & 0x7fffffu], v1 = Dv[x1 & 0x7fffffu], v2 = Dv[x2 & 0x7fffffu],
                             v3 = Dv[x3 & 0x7fffffu];
