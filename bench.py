@@ -41,7 +41,7 @@ MEASURED_TRAFFIC = {"mixed": 80.06e6 + 29.98e6, "fp64": 80.23e6 + 34.77e6}
 # (sm__pipe_fp64_cycles_active, share of active cycles), captured on the
 # first 16,384 cells of the default workload (a full launch is too long for
 # a multi-pass capture).
-MEASURED_FP64_PIPE = {"mixed": 0.597, "fp64": 0.805}
+MEASURED_FP64_PIPE = {"mixed": 0.568, "fp64": 0.873}
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12   # SMs x DFMA/clk x 2 x max clock
 FP64_PEAK_PROBE_TFLOPS = 1.193                    # DFMA timing probe on this GPU model
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12  # SMs x FFMA/clk x 2 x max clock
