@@ -180,6 +180,7 @@ struct HostTables {
         std::vector<int> j_d;
         std::vector<double> j_c;
     } lay[kLayouts];
+    float step_K = 0.f;
     int nD = 0, nD_F1 = 0, nD_1 = 0, nD_F2 = 0, nD_2 = 0, nJ = 0, nJ_nz = 0, n_items = 0, ntb = 0;
 };
 
@@ -253,28 +254,39 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
             for (int i = 0; i <= 5; ++i) cf[5 + i] = (float)c[i];
         }
     // the most by which a species' energy can change per kelvin of the
-    // temperature recovery's bracket: its largest c_v, sampled, a part in a
-    // thousand for what lies between the samples, and the step between the
-    // ranges over one kelvin
+    // temperature recovery's bracket, its largest c_v (from the expansion of
+    // the polynomial about the middle of every 20 K; a part in a thousand for
+    // the recovery's FP32 sums), and the kelvins of it that the largest step
+    // between the ranges at t_mid makes
     t.cv_max.resize(ns);
+    double step_K = 0.0;
     for (int s = 0; s < ns; ++s) {
         auto poly = [&](int rg) { return &t.tpoly[((size_t)s * 2 + rg) * kTpolyStride]; };
+        const double tm = d->t_mid[s];
+        constexpr double half = 10.0;
         double top = 0.0;
-        for (int Ti = (int)kTlo; Ti <= (int)kThi; Ti += 20)
-            for (int rg = 0; rg < 2; ++rg) {
-                if (rg == 0 ? Ti > d->t_mid[s] + 20 : Ti < d->t_mid[s] - 20) continue;
-                const double *c = poly(rg) + 6;
-                top = std::max(top, std::fabs((((c[4] * Ti + c[3]) * Ti + c[2]) * Ti + c[1]) * Ti + c[0]));
+        for (int rg = 0; rg < 2; ++rg) {
+            const double from = rg ? std::max(kTlo, tm) : kTlo, to = rg ? kThi : std::min(kThi, tm);
+            for (double T = from; T < to; T += 2 * half) {
+                double c[5];
+                std::copy(poly(rg) + 6, poly(rg) + 11, c);
+                for (int i = 0; i < 4; ++i)
+                    for (int j = 3; j >= i; --j) c[j] += (T + half) * c[j + 1];
+                double most = 0.0;
+                for (int i = 4; i >= 0; --i) most = most * half + std::fabs(c[i]);
+                top = std::max(top, most);
             }
-        const double T = d->t_mid[s];
+        }
         double step = 0.0;
-        if (T >= kTlo && T <= kThi)
+        if (tm >= kTlo && tm <= kThi)
             for (int rg = 0; rg < 2; ++rg) {
                 const double *c = poly(rg);
-                step += (rg ? 1 : -1) * (((((c[5] * T + c[4]) * T + c[3]) * T + c[2]) * T + c[1]) * T + c[0]);
+                step += (rg ? 1 : -1) * (((((c[5] * tm + c[4]) * tm + c[3]) * tm + c[2]) * tm + c[1]) * tm + c[0]);
             }
-        t.cv_max[s] = (float)(1.001 * top + std::fabs(step));
+        t.cv_max[s] = (float)(1.001 * top);
+        step_K = std::max(step_K, std::fabs(step) / top);
     }
+    t.step_K = (float)(1.001 * step_K + 0.01);
     // dense stoichiometry
     std::vector<int> nuR((size_t)nr * ns, 0), nuP((size_t)nr * ns, 0);
     for (int r = 0; r < nr; ++r)
@@ -724,6 +736,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
     m.tpoly = (const double *)at(i_tp);
     m.tpoly_f = (const float *)at(i_tpf);
     m.cv_max = (const float *)at(i_cvm);
+    m.step_K = t.step_K;
     m.sp = (const double *)at(i_sp);
     m.rxn_d = (const double *)at(i_rd);
     m.rxn_f = (const int *)at(i_rf);

@@ -132,10 +132,12 @@ struct DeviceMech {
     int nJ;                     // Jacobian entries gathered: ns*ns (species rows and columns)
     int nJ_nz;                  //   of which the first nJ_nz have reaction terms (longest list first)
     int n_items;                // species-gather work items
+    float step_K;               // kelvins of cv_max that an energy's step at t_mid makes, at
+                                //   most, and 0.01 on top
     const double *thermo;       // [16][2][ns] (coefficient-major, above)
     const double *tmid;         // [ns] (positive: compared as integers)
     const double *tpoly;        // [12][2][ns] energy and heat-capacity polynomials
-    const float *cv_max;        // [ns] bound of c_v on [kTlo, kThi] (HostTables)
+    const float *cv_max;        // [ns] bound of c_v on [kTlo, kThi]
     const float *tpoly_f;       // [12][2][ns] heat-capacity and energy polynomials in FP32
     const double *sp;           // [ns][4]
     const double *rxn_d;        // [nr][4] ln A (SI), beta, E/R, sum nu

@@ -414,11 +414,12 @@ __device__ __forceinline__ float wide_dotf(float a, float b, int cnt, float firs
 // passes to find that out: 36 species, mixed, 4 % of the recoveries took two
 // thirds of the passes.  So once a Newton step leaves the bracket, the
 // residual is held against the most that it can change over the bracket,
-// `slope` = sum |rho_s| max c_v,s (the energies' steps at t_mid included)
-// times its width: a larger one keeps its sign, and the passes would have
-// ended at the bracket's end, as this does.  (A hundredth of the width and of
-// a kelvin on top keep later Newton steps from ending inside the bracket
-// first: none could be below 0.01 K.)
+// `slope` = sum |rho_s| max c_v,s times the bracket's width and, however
+// narrow it is, times the kelvins step_K that the energies' steps at t_mid
+// are worth: a larger one keeps its sign, and the passes would have ended at
+// the bracket's end, as this does.  (A hundredth of the width and of a kelvin
+// on top keep later Newton steps from ending inside the bracket first: none
+// could be below 0.01 K.)
 //   The energies come from the multiplied-out polynomials (five DFMA per
 // species, no 1/T); with F32 the derivative sum c_v is formed in FP32, which
 // changes the Newton steps by a relative 1e-7 and not the root.  Without, a
@@ -568,7 +569,7 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
                 slope = Grp<G>::sum(slope);
             }
             // (infinities and NaN compare false)
-            if (left && fabsf(d2f_rz(f)) > slope * fmaf(1.01f, d2f_rz(hi) - d2f_rz(lo), 0.01f)) done = true;
+            if (left && fabsf(d2f_rz(f)) > slope * fmaf(1.01f, d2f_rz(hi) - d2f_rz(lo), m.step_K)) done = true;
         }
     }
     if (need) T_out = T;
