@@ -181,6 +181,7 @@ struct HostTables {
         std::vector<double> j_c;
     } lay[kLayouts];
     float step_K = 0.f;
+    double kink_lo = HUGE_VAL, kink_hi = 0.0;
     int nD = 0, nD_F1 = 0, nD_1 = 0, nD_F2 = 0, nD_2 = 0, nJ = 0, nJ_nz = 0, n_items = 0, ntb = 0;
 };
 
@@ -285,6 +286,18 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
             }
         t.cv_max[s] = (float)(1.001 * top);
         step_K = std::max(step_K, std::fabs(step) / top);
+        // a kink: c_v changes by more than a millionth, or the energy by more
+        // than the recovery's tolerance, above rounding (the 64 species of the
+        // largest mechanism here: 3e-16 and 1e-14 T)
+        auto cv = [&](int rg) {
+            const double *c = poly(rg) + 6;
+            return (((c[4] * tm + c[3]) * tm + c[2]) * tm + c[1]) * tm + c[0];
+        };
+        if (tm >= kTlo && tm <= kThi &&
+            (std::fabs(cv(1) - cv(0)) > 1e-6 * cv(0) || std::fabs(step) > kTtol * tm * cv(0))) {
+            t.kink_lo = std::min(t.kink_lo, tm * (1 - 2e-6));
+            t.kink_hi = std::max(t.kink_hi, tm * (1 + 2e-6));
+        }
     }
     t.step_K = (float)(1.001 * step_K + 0.01);
     // dense stoichiometry
@@ -737,6 +750,8 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
     m.tpoly_f = (const float *)at(i_tpf);
     m.cv_max = (const float *)at(i_cvm);
     m.step_K = t.step_K;
+    m.kink_lo = t.kink_lo;
+    m.kink_hi = t.kink_hi;
     m.sp = (const double *)at(i_sp);
     m.rxn_d = (const double *)at(i_rd);
     m.rxn_f = (const int *)at(i_rf);

@@ -74,9 +74,9 @@ __global__ void __launch_bounds__(kFieldThreads) state_from_tpy_kernel(DeviceMec
 // a guess, and where no density is negative (so that e(T) is increasing and
 // has one root), Newton runs in FP32 first, at a sixty-fourth of the cost: from
 // 1500 K the FP64 iterations were six or seven, from there they are two.
-// Bound by the FP64 pipe: after a step below a millionth of T the derivative
-// is kept (it has changed by as much, and the next step is below 1e-12 T), so
-// that the last iteration evaluates the energies alone.
+// Bound by the FP64 pipe: after a step below a millionth of T that is near no
+// kink the derivative is kept (it has changed by as much, and the next step is
+// below 1e-12 T), so that the last iteration evaluates the energies alone.
 // 524,365 cells of 36 species: 6.4 ms with c_p/R and h/RT re-read from L2 and
 // the FP64 iterations from 1500 K, 0.81 ms without, 0.70 ms with one
 // derivative.
@@ -133,6 +133,7 @@ __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m
 #pragma unroll 1
     for (int it = 1; it <= kTmaxIter; ++it) {
         const long long Tb = __double_as_longlong(T);
+        const bool kink = near_kink(m, T);
         double f = 0.0;
         if (near) {
 #pragma unroll 2
@@ -166,13 +167,13 @@ __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m
             lo = T;
         double Tn = fma(-f, slope, T), dT = Tn - T;
         const bool inside = Tn > lo && Tn < hi;
-        const double tol = (inside ? kTstep : kTtol) * T;
+        const double tol = (inside && !kink ? kTstep : kTtol) * T;
         // (a step below half an ulp leaves T at an end of the bracket)
         if (!inside && !(fabs(dT) <= tol)) {
             Tn = 0.5 * (lo + hi);
             dT = Tn - T;
         }
-        near = inside && fabs(dT) <= 1e-6 * T;
+        near = inside && !kink && fabs(dT) <= 1e-6 * T;
         T = Tn;
         if (fabs(dT) <= tol) {
             ok = !(T <= kTlo * (1.0 + 1e-9) || T >= kThi * (1.0 - 1e-9));

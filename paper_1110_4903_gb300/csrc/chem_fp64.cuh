@@ -117,5 +117,11 @@ __device__ __forceinline__ double frcp1(double a, const Fp64Ops &op) {
 __device__ __forceinline__ int thermo_range(const DeviceMech &m, int s, long long Tbits) {
     return Tbits > __ldg(reinterpret_cast<const long long *>(m.tmid) + s) ? 1 : 0;
 }
+// whether a small step of the temperature recovery from T may cross a t_mid
+// at which an energy or a heat capacity changes: the derivative is then
+// another range's, off by as much as the heat capacity changes
+__device__ __forceinline__ bool near_kink(const DeviceMech &m, double T) {
+    return bits_gt(T, m.kink_lo) & bits_lt(T, m.kink_hi);
+}
 
 }  // namespace chem

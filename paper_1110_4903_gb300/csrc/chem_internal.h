@@ -22,6 +22,7 @@ constexpr double kThi = 6000.0;
 constexpr int kTmaxIter = 50;          // temperature-recovery iterations
 constexpr double kTtol = 1e-13;        // |dT| <= kTtol * T ends the recovery,
 constexpr double kTstep = 1e-9;        //   a Newton step inside the bracket at kTstep * T
+                                       //   unless it may cross a kink (DeviceMech)
 
 // Polynomial tables are stored coefficient-major, so that the lanes of a
 // warp, which hold consecutive species, read consecutive words: coefficient
@@ -162,6 +163,10 @@ struct DeviceMech {
     const float *rxn_df;        // [nr][4] beta, Ea/R, sum nu, 0
     const float *d_cef;         // [nD] alpha - 1 in FP32
     const float *spf;           // [ns][4] M, 1/M, R/M, e_f in FP32
+    // the temperatures from which a step of a millionth may cross a kink, a
+    // t_mid at which some species' energy or heat capacity changes (infinity
+    // and 0: there is none)
+    double kink_lo, kink_hi;
 };
 
 struct StepOptions {

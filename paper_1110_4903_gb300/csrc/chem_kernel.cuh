@@ -404,8 +404,10 @@ __device__ __forceinline__ float wide_dotf(float a, float b, int cnt, float firs
 // Newton on sum_s rho_s e_s^sens(T) = e, safeguarded by bisection on
 // [kTlo, kThi] (Eq. 3 with the kinetic energy left to the flux stage).  A
 // Newton step of at most kTstep T ends it: with the derivative good to 1e-7
-// the temperature is then good to 1e-16, and another pass would only confirm
-// that.  Uniform across the warp.
+// (c_v changes by less than a millionth at a t_mid that is no kink) the
+// temperature is then good to 1e-15, and another pass would only confirm that.
+// A step from near a kink, which may cross it with the other side's
+// derivative, ends it at kTtol T.  Uniform across the warp.
 //   `cold` slots have no guess: where no density is negative (so that e(T) is
 // increasing and has one root) three Newton steps in FP32 find one, from
 // which two FP64 passes suffice instead of six.
@@ -423,10 +425,10 @@ __device__ __forceinline__ float wide_dotf(float a, float b, int cnt, float firs
 //   The energies come from the multiplied-out polynomials (five DFMA per
 // species, no 1/T); with F32 the derivative sum c_v is formed in FP32, which
 // changes the Newton steps by a relative 1e-7 and not the root.  Without, a
-// slot whose last step was below a millionth of T keeps its derivative (it
-// has changed by no more than that, and the step after is below 1e-12 T), and
-// a pass of such slots forms the energies alone: 2^19 cells of 9 species 26.8
-// -> 26.3 ms.
+// slot whose last step was below a millionth of T and near no kink keeps its
+// derivative (it has changed by no more than that, and the step after is below
+// 1e-12 T), and a pass of such slots forms the energies alone: 2^19 cells of 9
+// species 26.8 -> 26.3 ms.
 template <int G, int G0, bool F32>
 __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab, const double *x, int sl, bool need,
                                           bool cold, double guess, double &T_out, bool &ok) {
@@ -482,6 +484,9 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
     for (int it = 1; it <= kTmaxIter; ++it) {
         if (!__any_sync(kFull, !done)) break;
         const bool slopes = F32 || __any_sync(kFull, !done && !near);
+        // (FP64: in front of the sums, 2^20 cells of 9 species 51.8 ms, behind
+        // them 52.2; mixed behind them, 2^18 of 36 species 354.1 and 358.7 ms)
+        bool kink = !F32 && near_kink(m, T);
         const long long Tb = __double_as_longlong(T);
         const float Tf = F32 ? d2f_rz(T) : 0.f;
         double f = 0.0, fp = 0.0, xs = 0.0;
@@ -545,7 +550,8 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
                 // (comparisons of non-negative doubles on their bit patterns)
                 double Tn = fma(-f, rfp, T), dT = op.sub(Tn, T);
                 const bool inside = bits_gt(Tn, lo) && bits_lt(Tn, hi);
-                const double tol = (inside ? kTstep : kTtol) * T;
+                if (F32) kink = inside && near_kink(m, T);
+                const double tol = (inside && !kink ? kTstep : kTtol) * T;
                 // (a step below half an ulp leaves T at an end of the bracket:
                 // it ends the recovery, bisecting would start it all over)
                 if (!inside && bits_gt(fabs(dT), tol)) {
@@ -553,7 +559,7 @@ __device__ __forceinline__ void recover_T(const DeviceMech &m, const double *tab
                     dT = op.sub(Tn, T);
                     left = true;
                 }
-                if (!F32) near = inside && !bits_gt(fabs(dT), 1e-6 * T);
+                if (!F32) near = inside && !kink && !bits_gt(fabs(dT), 1e-6 * T);
                 T = Tn;
                 if (!bits_gt(fabs(dT), tol)) {
                     done = true;

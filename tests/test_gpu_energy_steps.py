@@ -96,3 +96,26 @@ def test_energy_inside_a_step(torch, step, n, mixed):
         # (the recovery halves its bracket down to 1e-13 T)
         for t in (T, field, oo["T"]):
             assert np.abs(t / 1000.0 - 1.0).max() < 1e-12
+
+
+# a heat capacity that changes by a part in 10^5 to a half at T_mid (the
+# energy continuous there), and energies that step by less than a millikelvin:
+# a last Newton step that crosses T_mid is no better than those differences
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("step,jump", [(0.0, 0.5), (0.0, -0.3), (0.0, 0.05), (0.0, 1e-5), (1e-7, 0.0), (2e-4, 0.0)])
+def test_last_steps_across_t_mid(torch, step, jump, mixed):
+    from paper_1110_4903_gb300 import chem
+    st = Stepped(step=step, jump=jump)
+    rng = np.random.default_rng(6)
+    n = 6000
+    rho = st.densities(n, 7)
+    # to either side of T_mid by up to 2e-6 of it, guessed from as near
+    sign = rng.choice([-1.0, 1.0], n)
+    T0 = 1000.0 + sign * 10.0 ** rng.uniform(-8.0, -2.7, n)
+    guess = 1000.0 - sign * 10.0 ** rng.uniform(-8.0, -2.7, n)
+    e = (rho * st.energies(T0)).sum(0).astype(np.float64)
+    for g in (guess, None):
+        T, status, field = temperatures(torch, st, rho, e, g, chem.MIXED if mixed else chem.FP64)
+        assert (status == 0).all()
+        # (the energy's rounding over its slope, and the recovery's own 1e-13 T)
+        assert np.abs(T / T0 - 1.0).max() < 1e-12 and np.abs(field / T0 - 1.0).max() < 1e-12
