@@ -65,7 +65,8 @@ static int validate(const chem_mech_desc *d) {
             if (!std::isfinite(d->nasa7[s * 14 + j]))
                 return fail(CHEM_E_BAD_MECHANISM, "species %d: NASA-7 coefficient %d not finite", s, j);
         // cp/R > 1 (cv > 0) on the temperature-recovery bracket keeps e(T)
-        // strictly increasing, so the recovery has one root
+        // strictly increasing within a range, so the recovery has one root
+        // (two at most where the energy steps down at t_mid)
         for (int Ti = (int)kTlo; Ti <= (int)kThi; ++Ti) {
             const double T = Ti;
             const double *a = d->nasa7 + s * 14 + (T > d->t_mid[s] ? 7 : 0);
@@ -182,6 +183,7 @@ struct HostTables {
     } lay[kLayouts];
     float step_K = 0.f;
     double kink_lo = HUGE_VAL, kink_hi = 0.0;
+    int one_root = 1;
     int nD = 0, nD_F1 = 0, nD_1 = 0, nD_F2 = 0, nD_2 = 0, nJ = 0, nJ_nz = 0, n_items = 0, ntb = 0;
 };
 
@@ -297,6 +299,7 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
             (std::fabs(cv(1) - cv(0)) > 1e-6 * cv(0) || std::fabs(step) > kTtol * tm * cv(0))) {
             t.kink_lo = std::min(t.kink_lo, tm * (1 - 2e-6));
             t.kink_hi = std::max(t.kink_hi, tm * (1 + 2e-6));
+            if (step < -kTtol * tm * cv(0)) t.one_root = 0;
         }
     }
     t.step_K = (float)(1.001 * step_K + 0.01);
@@ -752,6 +755,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
     m.step_K = t.step_K;
     m.kink_lo = t.kink_lo;
     m.kink_hi = t.kink_hi;
+    m.one_root = t.one_root;
     m.sp = (const double *)at(i_sp);
     m.rxn_d = (const double *)at(i_rd);
     m.rxn_f = (const int *)at(i_rf);

@@ -119,3 +119,19 @@ def test_last_steps_across_t_mid(torch, step, jump, mixed):
         assert (status == 0).all()
         # (the energy's rounding over its slope, and the recovery's own 1e-13 T)
         assert np.abs(T / T0 - 1.0).max() < 1e-12 and np.abs(field / T0 - 1.0).max() < 1e-12
+
+
+# energies that step down at T_mid leave two temperatures to an energy near
+# there: the answer is the upper one, which the FP64 iterations meet first on
+# their way down from 1500 K, also within a rounding of FP32 above T_mid
+def test_energy_steps_down(torch):
+    from paper_1110_4903_gb300 import chem
+    st = Stepped(step=-1.0)
+    rng = np.random.default_rng(8)
+    for n in (240, 6000):
+        rho = st.densities(n, 9)
+        T0 = 1000.0 + 10.0 ** rng.uniform(-7.0, -1.0, n)
+        e = (rho * st.energies(T0)).sum(0).astype(np.float64)
+        T, status, field = temperatures(torch, st, rho, e, None, chem.FP64)
+        assert (status == 0).all()
+        assert np.abs(T / T0 - 1.0).max() < 1e-12 and np.abs(field / T0 - 1.0).max() < 1e-12
