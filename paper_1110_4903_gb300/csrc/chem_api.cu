@@ -354,6 +354,11 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
     struct DEnt { int r, k, grp; int fa, fb, ba, bb, vf, vb; double alpha1; };
     std::vector<DEnt> ents;
     for (int r = 0; r < nr; ++r) {
+        // (none of a reaction that changes nothing: the FP32 gather's missing
+        // terms are a zero times D entry 0, which may be infinite or NaN only
+        // where the Jacobian is as well)
+        const size_t row = (size_t)r * ns;
+        if (std::equal(nuR.begin() + row, nuR.begin() + row + ns, nuP.begin() + row)) continue;
         std::vector<int> cols;
         auto addc = [&](int s) { if (std::find(cols.begin(), cols.end(), s) == cols.end()) cols.push_back(s); };
         for (int j = 0; j < 3; ++j) if (d->reac_sp[r * 3 + j] >= 0) addc(d->reac_sp[r * 3 + j]);
