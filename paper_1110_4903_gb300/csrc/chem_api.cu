@@ -1152,7 +1152,9 @@ int chem_advance_segmented(chem_handle_t hh, const chem_advance_args *a, int64_t
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing((cudaStream_t)a->stream, &cap);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamIsCapturing");
-    const bool chained = cap == cudaStreamCaptureStatusNone;
+    // (with rows closer together than the cells are many, segments share
+    // elements: they run one after another)
+    const bool chained = cap == cudaStreamCaptureStatusNone && ld >= a->n_cells;
     LaunchChain chain;
     const int64_t slots = (int64_t)cfg->grid * (cfg->block / 32) * (32 / G);
     chain.max_wpb = segment_cells <= 4 * slots ? 1 : 0;
