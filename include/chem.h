@@ -381,8 +381,8 @@ int chem_server_stats(chem_server_t s, chem_server_stats_t *out);
  *                       equal to the scalar elimination to rounding.
  *   CHEM_LU_ONCHIP      A[(k*n + i)*n + j], b[k*n + i] (contiguous); 8 to 256
  *                       threads per system, the matrix in shared memory
- *                       (CHEM_E_UNSUPPORTED when n*(n+1) doubles do not
- *                       fit); factors and pivots bit for bit as
+ *                       (CHEM_E_UNSUPPORTED beyond n = 169, whose
+ *                       n*((n+2)|1) doubles are the most that fit); factors and pivots bit for bit as
  *                       CHEM_LU_GLOBAL, x to rounding (the back
  *                       substitution runs by columns across the threads).
  * Device pointers; asynchronous on `stream`; CHEM_E_INVALID_ARG for an

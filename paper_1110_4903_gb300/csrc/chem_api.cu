@@ -913,9 +913,9 @@ int launch_cfg(Handle *h, const chem_advance_args *a, int prec, const LaunchCfg 
     // does not fill the resident warps is spread evenly over the SMs: the
     // blocks an SM gets hold its share of the warps, not as many warps as
     // fit.  Full blocks of 10 warps put 1,024 cells of 36 species on 103 SMs
-    // (11.9 ms, mixed); blocks of 7 warps on 147 SMs take 10.3 ms, and
-    // 1,024 cells of 9 species on 128 SMs instead of 13 take 0.58 instead of
-    // 0.78 ms (FP64).  Blocks of one warp are not dealt out evenly (13.7 ms).
+    // (8.5 ms, mixed); blocks of 7 warps on 147 SMs take 6.4 ms.  8,192 cells
+    // of 9 species take 1.43 and 1.30 ms (FP64).  Blocks of one warp are not
+    // dealt out evenly (an earlier kernel: 13.7 ms against 10.3).
     //   With several cells per warp, a call of at most one and a half cells
     // per resident warp (two blocks per SM) starts with one to a warp, and any
     // other ends so (wide warps, be_kernel).  152 SMs, 9 species, eight cells
@@ -950,7 +950,10 @@ int launch_cfg(Handle *h, const chem_advance_args *a, int prec, const LaunchCfg 
     lc.blockDim = dim3((unsigned)wpb * 32);
     lc.dynamicSmemBytes = smem;
     lc.stream = st;
-    // what the blocks do not need of the SM's shared memory serves as L1
+    // what the blocks do not need of the SM's shared memory serves as L1.  (A
+    // small call on another stream finds less room so, but two calls of 1,024
+    // cells of 36 species on two streams take 7.8 ms, mixed, one alone 6.4;
+    // full blocks with the largest carveout took 12.5 and 12.0.)
     cudaLaunchAttribute at[2]{};
     at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
     const long long sm_smem = h->max_smem_optin + 1024;

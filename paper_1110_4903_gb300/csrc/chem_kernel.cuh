@@ -2141,7 +2141,7 @@ __device__ __forceinline__ void step_cells(const DeviceMech &m, const StepOption
 
 // At most 10 warps per block and 96 registers per thread: 20 warps fit on an
 // SM when shared memory allows it (2 blocks of 10; the mixed path at 36
-// species, 11.3 KB per cell).
+// species, 11.5 KB per cell).
 //   Wide warps: with several cells per warp, an iteration is a serial chain
 // that takes a warp as long for one cell as for all (4 lanes per cell, 9
 // species, alone on its SM: 89,000 cycles mixed, 152,000 FP64), and the last
