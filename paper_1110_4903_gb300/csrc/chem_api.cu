@@ -183,7 +183,7 @@ struct HostTables {
     } lay[kLayouts];
     float step_K = 0.f;
     double kink_lo = HUGE_VAL, kink_hi = 0.0;
-    int one_root = 1;
+    int fp32_start = 1;
     int nD = 0, nD_F1 = 0, nD_1 = 0, nD_F2 = 0, nD_2 = 0, nJ = 0, nJ_nz = 0, n_items = 0, ntb = 0;
 };
 
@@ -299,7 +299,11 @@ static void build_tables(const chem_mech_desc *d, HostTables &t) {
             (std::fabs(cv(1) - cv(0)) > 1e-6 * cv(0) || std::fabs(step) > kTtol * tm * cv(0))) {
             t.kink_lo = std::min(t.kink_lo, tm * (1 - 2e-6));
             t.kink_hi = std::max(t.kink_hi, tm * (1 + 2e-6));
-            if (step < -kTtol * tm * cv(0)) t.one_root = 0;
+            // (down: two temperatures to an energy; up by a thousandth of T:
+            // Newton to and fro across the step may take all of the
+            // recovery's passes, and which cells it fails is a matter of
+            // where it starts)
+            if (step < -kTtol * tm * cv(0) || step > 1e-3 * tm * cv(0)) t.fp32_start = 0;
         }
     }
     t.step_K = (float)(1.001 * step_K + 0.01);
@@ -760,7 +764,7 @@ static int upload(const HostTables &t, int ns, int nr, Handle *h) {
     m.step_K = t.step_K;
     m.kink_lo = t.kink_lo;
     m.kink_hi = t.kink_hi;
-    m.one_root = t.one_root;
+    m.fp32_start = t.fp32_start;
     m.sp = (const double *)at(i_sp);
     m.rxn_d = (const double *)at(i_rd);
     m.rxn_f = (const int *)at(i_rf);

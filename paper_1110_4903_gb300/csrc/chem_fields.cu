@@ -71,10 +71,10 @@ __global__ void __launch_bounds__(kFieldThreads) state_from_tpy_kernel(DeviceMec
 
 // Temperature of (rho, e): Newton on sum_s rho_s e_s^sens(T) = e safeguarded by
 // bisection on [kTlo, kThi], ended as in the step.  Without a guess, and where
-// no density is negative and no energy steps down at a t_mid (so that e(T) is
-// increasing and has one root), Newton runs in FP32 first, at a sixty-fourth
-// of the cost: from 1500 K the FP64 iterations were six or seven, from there
-// they are two.
+// no density is negative and no energy steps down at a t_mid or far up (so
+// that e(T) is increasing and has one root), Newton runs in FP32 first, at a
+// sixty-fourth of the cost: from 1500 K the FP64 iterations were six or seven,
+// from there they are two.
 // Bound by the FP64 pipe: after a step below a millionth of T that is near no
 // kink the derivative is kept (it has changed by as much, and the next step is
 // below 1e-12 T), so that the last iteration evaluates the energies alone.
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kFieldThreads) temperature_kernel(DeviceMech m
     double lo = kTlo, hi = kThi, T = Tg ? Tg[i] : 1500.0;
     if (!(T > lo && T < hi)) T = 1500.0;
     const double ei = e[i];
-    if (!Tg && nonneg && m.one_root) {
+    if (!Tg && nonneg && m.fp32_start) {
         const float ef = d2f_rz(ei);
         float Tf = 1500.f;
 #pragma unroll 1

@@ -167,7 +167,7 @@ struct DeviceMech {
     // t_mid at which some species' energy or heat capacity changes (infinity
     // and 0: there is none)
     double kink_lo, kink_hi;
-    int one_root;               // no species' energy steps down at its t_mid
+    int fp32_start;             // no species' energy steps down at its t_mid, or far up
 };
 
 struct StepOptions {

@@ -408,10 +408,10 @@ __device__ __forceinline__ float wide_dotf(float a, float b, int cnt, float firs
 // temperature is then good to 1e-15, and another pass would only confirm that.
 // A step from near a kink, which may cross it with the other side's
 // derivative, ends it at kTtol T.  Uniform across the warp.
-//   `cold` slots have no guess, and no energy steps down at a t_mid: where no
-// density is negative either (so that e(T) is increasing and has one root)
-// three Newton steps in FP32 find one, from which two FP64 passes suffice
-// instead of six.
+//   `cold` slots have no guess, and no energy steps down at a t_mid, or up by
+// a thousandth of it: where no density is negative either (so that e(T) is
+// increasing and has one root) three Newton steps in FP32 find one, from which
+// two FP64 passes suffice instead of six.
 //   A diverging substep's densities, some negative and large, often have no
 // temperature, and halving the bracket down to one of its ends takes up to 48
 // passes to find that out: 36 species, mixed, 4 % of the recoveries took two
@@ -1981,7 +1981,7 @@ __device__ __forceinline__ void step_cells(const DeviceMech &m, const StepOption
             if (!__any_sync(kFull, needT || act != kNoAction)) break;
             double Tr = T;
             bool ok = false;
-            recover_T<G, G0, sizeof(JT) == 4>(m, tab, sm.x, sl, needT, state == kInitT && (Q || !b.T_in) && m.one_root, T,
+            recover_T<G, G0, sizeof(JT) == 4>(m, tab, sm.x, sl, needT, state == kInitT && (Q || !b.T_in) && m.fp32_start, T,
                                               Tr, ok);
             int neg = 0;
             if (__any_sync(kFull, state == kCheckT)) {

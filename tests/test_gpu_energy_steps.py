@@ -135,3 +135,22 @@ def test_energy_steps_down(torch):
         T, status, field = temperatures(torch, st, rho, e, None, chem.FP64)
         assert (status == 0).all()
         assert np.abs(T / T0 - 1.0).max() < 1e-12 and np.abs(field / T0 - 1.0).max() < 1e-12
+
+
+# where an energy steps by more than a thousandth of T, up or down, no guess
+# is the guess 1500 K: also within a thousandth of the step's ends, where the
+# recovery's passes may not suffice
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("step", [-20.0, 2.0, 20.0, 100.0])
+def test_no_guess_is_the_plain_start(torch, step, mixed):
+    from paper_1110_4903_gb300 import chem
+    st = Stepped(step=step)
+    rng = np.random.default_rng(12)
+    n = 60000
+    rho = st.densities(n, 13)
+    lo, hi = ((rho * st.energies(np.full(n, 1000.0), side)).sum(0) for side in (0, 1))
+    e = (lo + rng.uniform(0.0, 1.0, n) * (hi - lo)).astype(np.float64)
+    cold, warm = (temperatures(torch, st, rho, e, guess, chem.MIXED if mixed else chem.FP64)
+                  for guess in (None, np.full(n, 1500.0)))
+    for a, b in zip(cold, warm):
+        assert np.array_equal(a, b, equal_nan=True)
